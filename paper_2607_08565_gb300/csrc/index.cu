@@ -5,8 +5,8 @@
 // block hash, which tiers hold the block. One table serves all tiers: an
 // entry is the 64-bit block hash followed by W = ceil((N+1)/64) mask words,
 // bit i < N = local tier of instance i, bit N = global tier. Slots are grouped
-// in buckets of kSlots; a one-byte tag per slot (0 = empty, else 0x80 | low
-// 7 key bits) and the bucket's overflow count live in a separate 16-byte tag
+// in buckets of kSlots; a one-byte tag per slot (0 = empty, else the low key
+// byte, 1 for 0) and the bucket's overflow count live in a separate 16-byte tag
 // group, so that a lookup reads one tag group and then only the entry whose
 // tag matches. A key that leaves its last tier gives its slot back (the
 // primitives and their concurrency contract are in table.cuh), so a table
@@ -240,8 +240,7 @@ int smetric_index_create(const smetric_index_config* cfg, smetric_index** out) {
             cudaMalloc(&x->tags, tag_bytes) == cudaSuccess &&
             cudaMalloc(&x->status, sizeof(int32_t)) == cudaSuccess &&
             cudaMalloc(&x->block_off, (R + 1) * sizeof(int64_t)) == cudaSuccess &&
-            // two spare words: k_chain_probe copies a chunk's digests in whole 16-byte pieces
-            cudaMalloc(&x->digest, (max_blocks + 2) * sizeof(uint64_t)) == cudaSuccess &&
+            cudaMalloc(&x->digest, (max_blocks > 0 ? max_blocks : 1) * sizeof(uint64_t)) == cudaSuccess &&
             cudaMalloc(&x->hashes, (max_blocks > 0 ? max_blocks : 1) * sizeof(uint64_t)) == cudaSuccess &&
             cudaMalloc(&x->masks, (max_blocks > 0 ? max_blocks : 1) * W * sizeof(uint64_t)) == cudaSuccess &&
             // one per request-aligned 32-block chunk: at most max_blocks / 32 + R

@@ -15,21 +15,24 @@
 //                 request's group key (its first-block hash) into the group
 //                 table. (k_digest and k_digest_any cover block sizes the
 //                 tensor maps do not.)
-//   k_lead        one thread per request: whether it leads its group (the
-//                 group's lowest request index).
+//   k_lead        one warp per request: its group's leader (the group's lowest
+//                 request index), the shared prefix (leading blocks with the
+//                 leader's digests), and whether the chain kernel takes it.
 //   k_chain_probe one CTA per SM. Chain warps (one lane per request the CTA
-//                 owns) run the serial chain h_b over the digests and write
-//                 the session key; beside them, probe warps find each
-//                 member's shared prefix with its leader and probe every
-//                 block not shared: the tier masks of h_b from the index (16
-//                 tags of the home bucket, then the matching entry), and the
-//                 AND of each 32-block chunk's masks.
+//                 owns) run the serial chain h_b over the digests in a ring in
+//                 shared memory; beside them, probe warps fill the ring, write
+//                 the session keys (and the hashes, where wanted) and probe
+//                 every block not shared: the tier masks of h_b from the index
+//                 (15 tags of the home bucket, then the matching entry), and
+//                 the AND of each 32-block chunk's masks.
 //   k_walk        one warp per request walks the runs of the local tiers and
 //                 the global tier (a member over its leader's probes up to
 //                 its shared prefix), 32 chunks per step from the chunk ANDs
-//                 and block by block where a run ends; then lanes =
-//                 instances for the cost and a shuffle argmin with ties to
-//                 the lowest id (or one of the policy scores).
+//                 and block by block where a run ends; a short tail past the
+//                 shared prefix that the chain kernel left out is chained and
+//                 probed here; then lanes = instances for the cost and a
+//                 shuffle argmin with ties to the lowest id (or one of the
+//                 policy scores).
 
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -58,10 +61,8 @@ constexpr int kChunk = 32;        // blocks per digest task (one per lane)
 constexpr int kDigestWarps = 8;   // most warps per digest CTA
 constexpr int kTmaWarps = 24;     // warps per TMA digest CTA (two CTAs per SM)
 constexpr int kTmaStages = 1;     // copy stages per TMA digest warp
-constexpr int kChainThreads = 32;   // one warp per CTA: chains spread over every SM
-constexpr int kChainAhead = 16;   // digests prefetched per request
 constexpr int kMatchWarps = 8;    // warps per walk CTA
-constexpr int kGroupAhead = 8;    // 32-block rounds of hashes a group warp compares at once
+constexpr int kGroupAhead = 8;    // 32-block rounds of digests a group warp compares at once
 
 // ---------------------------------------------------------------------------
 // prep
@@ -191,12 +192,44 @@ __global__ void __launch_bounds__(1024) k_prep(const int64_t* __restrict__ off, 
 // ---------------------------------------------------------------------------
 
 // The group stage works from the digests, so that it needs no finished chain:
-// a request's first-block hash h_0 = chain step from h_init over d_0 is the
+// a request's first-block hash h_0 = chain_step(h_init, its first digest) is the
 // group key, and the shared-prefix length is the number of leading blocks
 // whose digests equal the leader's. Equal digests from equal previous hashes
 // give equal hashes, so the leader's masks serve those blocks exactly.
-__device__ __forceinline__ uint64_t first_hash(uint64_t h_init, uint64_t d0) {
-  uint64_t h = mix64((h_init + kGamma) ^ d0);
+//
+// A stored digest is d_b ^ (d_b >> 30): the chain's first xor-shift
+// x ^ (x >> 30) is linear over xor, so the digest's share of it is taken here,
+// off the chain's serial path (a bijection, so equal words are equal digests).
+__device__ __forceinline__ uint64_t stored_digest(uint64_t d) { return d ^ (d >> 30); }
+
+// h_b before the sentinel remap, from h_{b-1} and the stored digest of block b:
+// mix64((h_{b-1} + kGamma) ^ d_b) on 32-bit halves, for the serial chain where
+// only latency counts. The high word of each product is the low-by-low high
+// half plus the two cross products, the second accumulated onto the first.
+__device__ __forceinline__ uint64_t chain_raw(uint64_t hp, uint64_t ds) {
+  const uint64_t a = hp + kGamma;
+  uint32_t lo = (uint32_t)a, hi = (uint32_t)(a >> 32);
+  auto mul = [&](uint64_t c) {
+    const uint32_t cl = (uint32_t)c, ch = (uint32_t)(c >> 32);
+    const uint32_t x = hi * cl + lo * ch;
+    hi = __umulhi(lo, cl) + x;
+    lo = lo * cl;
+  };
+  auto xs = [&](int n, uint32_t xl, uint32_t xh) {
+    lo ^= __funnelshift_r(lo, hi, n) ^ xl;
+    hi ^= (hi >> n) ^ xh;
+  };
+  xs(30, (uint32_t)ds, (uint32_t)(ds >> 32));
+  mul(0xBF58476D1CE4E5B9ull);
+  xs(27, 0, 0);
+  mul(0x94D049BB133111EBull);
+  xs(31, 0, 0);
+  return ((uint64_t)hi << 32) | lo;
+}
+
+// One chain step with the sentinel remap.
+__device__ __forceinline__ uint64_t chain_step(uint64_t hp, uint64_t ds) {
+  const uint64_t h = chain_raw(hp, ds);
   return h < 2 ? (h | 2) : h;
 }
 
@@ -367,9 +400,9 @@ __global__ void __launch_bounds__(kDigestWarps * 32)
     if (cur.valid) {
       const int delta = (int)((cur.tok0 * 4) & 15);  // 0, 4, 8 or 12
       const uint64_t* row = reinterpret_cast<const uint64_t*>(st + lane * NP) + (delta >> 3);
-      const uint64_t d = digest_row<HB>(row, (delta & 4) != 0, HB, d_init);
+      const uint64_t d = stored_digest(digest_row<HB>(row, (delta & 4) != 0, HB, d_init));
       digest[c * kChunk + lane] = d;
-      if (groups && cur.head) group_insert(groups, gmask, first_hash(h_init, d), cur.req);
+      if (groups && cur.head) group_insert(groups, gmask, chain_step(h_init, d), cur.req);
     }
     __syncwarp();
     cur = nxt;
@@ -525,9 +558,9 @@ __global__ void __launch_bounds__(kTmaWarps * 32)
     if (vc) {
       const int delta = (int)((tc * 4) & 15);  // 0, 4, 8 or 12
       const uint64_t* row = reinterpret_cast<const uint64_t*>(stages + (size_t)s * STAGE + lane * ROW) + (delta >> 3);
-      const uint64_t d = digest_row<HB>(row, (delta & 4) != 0, HB, d_init);
+      const uint64_t d = stored_digest(digest_row<HB>(row, (delta & 4) != 0, HB, d_init));
       digest[gc] = d;
-      if (groups && hc) group_insert(groups, gmask, first_hash(h_init, d), rc);
+      if (groups && hc) group_insert(groups, gmask, chain_step(h_init, d), rc);
     }
     __syncwarp();
     if (c + STAGES * warps < c_hi) {
@@ -578,110 +611,12 @@ __global__ void __launch_bounds__(kDigestWarps * 32)
     const int64_t a = (4 * tok0) & ~(int64_t)15;
     for (int i = 0; i < nch; ++i) row[i] = load_piece(tb, a + 16 * i, token_bytes - (a + 16 * i));
     const int delta = (int)((tok0 * 4) & 15);
-    const uint64_t d = digest_row<0>(reinterpret_cast<const uint64_t*>(row) + (delta >> 3), (delta & 4) != 0,
-                                     B >> 1, d_init);
+    const uint64_t d = stored_digest(digest_row<0>(reinterpret_cast<const uint64_t*>(row) + (delta >> 3),
+                                                   (delta & 4) != 0, B >> 1, d_init));
     digest[f] = d;
-    if (groups && f == __ldg(block_off + r)) group_insert(groups, gmask, first_hash(h_init, d), r);
+    if (groups && f == __ldg(block_off + r)) group_insert(groups, gmask, chain_step(h_init, d), r);
   }
 }
-
-// ---------------------------------------------------------------------------
-// chain
-// ---------------------------------------------------------------------------
-
-// 32-byte global load (read-only path) and store of four 64-bit words; the
-// address must be 32-byte aligned.
-__device__ __forceinline__ void ld_nc_v4(const uint64_t* p, uint64_t (&v)[4]) {
-  asm volatile("ld.global.nc.v4.u64 {%0,%1,%2,%3}, [%4];\n"
-               : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3])
-               : "l"(p));
-}
-__device__ __forceinline__ void st_v4(uint64_t* p, uint64_t a, uint64_t b, uint64_t c, uint64_t d) {
-  asm volatile("st.global.v4.u64 [%0], {%1,%2,%3,%4};\n" ::"l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
-}
-
-// End of a request's chain: the session key is read back rather than tested
-// at every serial step.
-__device__ __forceinline__ void nb_done(int32_t r, int64_t nb, const uint64_t* hout, int64_t kS,
-                                        uint64_t* __restrict__ sk_out) {
-  sk_out[r] = nb > 0 ? hout[kS] : 0;
-}
-
-__global__ void __launch_bounds__(kChainThreads)
-    k_chain(const int64_t* __restrict__ off, const int64_t* __restrict__ block_off, int32_t n, int B,
-            int S, uint64_t h_init, const int32_t* __restrict__ batch_ok,
-            const uint64_t* __restrict__ digest, uint64_t* __restrict__ hashes,
-            uint64_t* __restrict__ sk_out) {
-  pdl_enter();
-  const int32_t r = blockIdx.x * kChainThreads + threadIdx.x;
-  if (r >= n) return;
-  if (!*batch_ok) { sk_out[r] = 0; return; }
-  const int64_t bo = block_off[r];
-  const int64_t nb = block_off[r + 1] - bo;
-  const uint64_t* const d = digest + bo;
-  uint64_t* const hout = hashes + bo;
-  const int64_t kS = (nb < S ? nb : S) - 1;
-  uint64_t h = h_init;
-  auto step = [](uint64_t hp, uint64_t db) {
-    uint64_t x = mix64_halves((hp + kGamma) ^ db);
-    if (x < 2) x |= 2;
-    return x;
-  };
-  // Digests are read and hashes written four blocks per 32-byte access (a
-  // lane's accesses are its own request's and do not coalesce across the
-  // warp, and fewer instructions shorten every serial step): single blocks
-  // up to a 32-byte boundary and after the last whole quad. A caller hash
-  // buffer in another 32-byte phase than the digests takes one block per
-  // access throughout.
-  if (((reinterpret_cast<uintptr_t>(d) ^ reinterpret_cast<uintptr_t>(hout)) & 31) != 0) {
-    for (int64_t k = 0; k < nb; ++k) {
-      h = step(h, __ldg(d + k));
-      hout[k] = h;
-    }
-    nb_done(r, nb, hout, kS, sk_out);
-    return;
-  }
-  int64_t b = 0;
-  while (b < nb && (reinterpret_cast<uintptr_t>(d + b) & 31)) {
-    h = step(h, __ldg(d + b));
-    hout[b] = h;
-    ++b;
-  }
-  const uint64_t* const dq = d + b;
-  uint64_t* const hq = hout + b;
-  const int64_t nq = (nb - b) >> 2;  // whole quads
-  constexpr int Q = kChainAhead / 4;
-  uint64_t c[Q][4], x[Q][4];
-#pragma unroll
-  for (int j = 0; j < Q; ++j)
-    if (j < nq) ld_nc_v4(dq + 4 * j, c[j]);
-  for (int64_t q0 = 0; q0 < nq; q0 += Q) {
-#pragma unroll
-    for (int j = 0; j < Q; ++j)
-      if (q0 + Q + j < nq) ld_nc_v4(dq + 4 * (q0 + Q + j), x[j]);
-#pragma unroll
-    for (int j = 0; j < Q; ++j) {
-      if (q0 + j < nq) {
-        const uint64_t a0 = step(h, c[j][0]), a1 = step(a0, c[j][1]), a2 = step(a1, c[j][2]);
-        h = step(a2, c[j][3]);
-        st_v4(hq + 4 * (q0 + j), a0, a1, a2, h);
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < Q; ++j)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) c[j][k] = x[j][k];
-  }
-  for (int64_t k = b + 4 * nq; k < nb; ++k) {
-    h = step(h, __ldg(d + k));
-    hout[k] = h;
-  }
-  nb_done(r, nb, hout, kS, sk_out);
-}
-
-// ---------------------------------------------------------------------------
-// group
-// ---------------------------------------------------------------------------
 
 // ---------------------------------------------------------------------------
 // match
@@ -704,8 +639,7 @@ __device__ __forceinline__ void probe_one(const uint8_t* __restrict__ tags, cons
     const uint4 tv = __ldg(reinterpret_cast<const uint4*>(tags + b * kBucket));
     uint32_t cand = slot_match(tv, tg);
     while (cand) {
-      const int sl = __ffs(cand) - 1;
-      cand &= cand - 1;
+      const int sl = next_slot(cand);
       const ulonglong2* e = reinterpret_cast<const ulonglong2*>(table + (b * kSlots + sl) * EW);
       ulonglong2 v[NV];
 #pragma unroll
@@ -725,176 +659,350 @@ __device__ __forceinline__ void probe_one(const uint8_t* __restrict__ tags, cons
 // chain, shared prefix and probe in one kernel
 // ---------------------------------------------------------------------------
 //
-// The chain is bound by the latency of its dependent mix64 steps and the
-// probe by random memory accesses, so one kernel runs both at once. One CTA
-// of 32 warps per SM; the SM deals a CTA's warps to its four schedulers in
-// turn (warp w to scheduler w mod 4). The chain warps (lane = request) are
-// warps 0 .. chain_warps - 1, one per scheduler, beside probe warps that
-// mostly wait on memory, so their dependent steps seldom wait for issue. The
-// other warps first find each request's group leader and shared prefix, then
-// probe the index for each 32-block chunk as soon as its chain has published
-// it.
+// The chain is bound by the latency of its dependent steps and the probe by
+// random memory accesses, so one kernel runs both at once: one CTA of
+// kCpWarps warps per SM. Chain warps (lane = request, warps 0 ..
+// chain_warps - 1, one per scheduler) only turn digests into hashes, in place
+// in a ring of 32-block chunks in shared memory; every other access is a probe
+// warp's. Why the ring: a chain step's own latency is ~75 cycles, any number
+// of chain warps up to one per scheduler, but ~147 with four chain warps that
+// store their hashes per lane to global memory (32 sectors an instruction).
+// Measured, N = 64, B = 32, 24k tokens a prompt: a step takes 88 cycles with few
+// requests an SM and ~140 beside the probes of 8,192 requests (before: 145 and
+// ~205); the kernel 31 us instead of 46 for 16 requests, 53 instead of 83 for
+// 777, 99 instead of 138 for 8,192 and 245 instead of 460 for 32,768, where
+// 6.4M probes at 29 G/s are what random reads allow.
 //
-// CTA c owns requests c, c + gridDim, c + 2 gridDim, ..., taken in groups of
-// up to 32 * chain_warps (one chain lane each). Chunk q of request r is its
-// blocks 32q .. 32q + 31; the chunk ANDs the walk reads are kept per such
+// Lane j of the CTA chains a stream of requests, one after another; position q
+// of the stream is a 32-block chunk of one of them, kept in slot q mod slots
+// of lane j's part of the ring. Item (q, j), taken by the probe warps in
+// position-major order: once the chain warp has chained position q, read its
+// hashes, put the digests of position q + slots into the slot, then probe the
+// index with the hashes, store masks and the chunk's AND, and (where wanted)
+// store the hashes, coalesced. Two mbarriers per chain warp and slot carry the
+// order: `full` (one arrival per lane in use) and `ready` (the chain warp's).
+// A slot's barriers cannot run ahead of an item that still waits, since its
+// own refill is one of the arrivals that the next phase needs; an item taken
+// more than `slots` positions ahead first polls the chain warp's position
+// counter, so that the parity it then waits for is that of its own phase.
+//
+// Chunk q of request r is its blocks 32q .. 32q + 31; the chunk ANDs the walk reads are kept per such
 // request-aligned chunk, at index chunk_off[r] + q.
 constexpr int kCpWarps = 32;
+constexpr int kHashWarps = 24;       // without an index; 8,192 prompts of 750 blocks: 109 us, with 32 warps 113, with 16 120
+__host__ __device__ constexpr int cp_warps(int W) { return W == 0 ? kHashWarps : kCpWarps; }
 constexpr int kCpMaxChainWarps = 4;  // warps 0 .. 3, one per scheduler
-constexpr int kCpMaxGroup = 32 * kCpMaxChainWarps;
-constexpr int kCpRingDigests = 34;   // a chunk's 32 digests and one neighbour on each side
-constexpr int kCpRingBytes = 560;    // two such slots per chain lane, in 16-byte pieces
-constexpr int kCpProbes = 2;         // chunks a probe warp takes at once (probes in flight per lane)
-constexpr int kCpDealMax = 512;      // requests a CTA can own when leaders are dealt out
+constexpr int kCpMaxLanes = 32 * kCpMaxChainWarps;
+// Bytes of a slot: 32 words, and 16 bytes that make the distance between the
+// lanes' rows of one slot an odd number of 16-byte units, so that a chain
+// warp's 16-byte accesses meet no bank conflict.
+constexpr int kCpRow = 272;
+constexpr int kCpMaxSlots = 8;       // 8 with one or two chain warps, 4 with more (139 KB of ring at most)
+constexpr int kCpRound = 512;        // requests a CTA takes at a time
 
-__device__ __forceinline__ int32_t ld_acquire_cta(const int32_t* p) {
-  int32_t v;
-  asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];\n" : "=r"(v) : "r"(smem_u32(p)) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_release_cta(int32_t* p, int32_t v) {
-  asm volatile("st.release.cta.shared::cta.s32 [%0], %1;\n" ::"r"(smem_u32(p)), "r"(v) : "memory");
-}
-// A chain hash another warp of this CTA has published (ordered by ld_acquire_cta).
-__device__ __forceinline__ uint64_t ld_relaxed_cta(const uint64_t* p) {
-  uint64_t v;
-  asm volatile("ld.relaxed.cta.global.u64 %0, [%1];\n" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-
-// One chain step: h_b from h_{b-1} and d_b, with the sentinel remap.
-__device__ __forceinline__ uint64_t chain_step(uint64_t hp, uint64_t db) {
-  uint64_t x = mix64_halves((hp + kGamma) ^ db);
-  if (x < 2) x |= 2;
-  return x;
+__device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(mbar) : "memory");
 }
 
-// Bounded wait until a shared counter exceeds v; false on timeout.
-__device__ __forceinline__ bool wait_above(const int32_t* p, int32_t v) {
+// Bounded poll until a chain warp's position counter reaches v (which only says
+// which phase its barriers are in: the barriers order the data); positions
+// take about a microsecond each, so the sleep grows with the distance.
+__device__ __forceinline__ bool poll_at_least(const int32_t* p, int32_t v, volatile int* failed) {
+  bool ok = false;
   for (uint32_t i = 0; i < kSpinLimit; ++i) {
-    if (ld_acquire_cta(p) > v) return true;
-    __nanosleep(256);  // a long sleep keeps waiting warps off the chain warps' schedulers
+    const int32_t at = *reinterpret_cast<const volatile int32_t*>(p);
+    ok = at >= v;
+    if (ok || ((i & 15) == 15 && *failed)) break;
+    __nanosleep(400u * (uint32_t)min(v - at, 8));
   }
-  return false;
+  ok = __all_sync(kFull, ok);
+  if (!ok) *failed = 1;
+  return ok;
 }
 
-// Tier masks of U keys at once: the home-bucket tags of all, then the first
-// tag match's entry of all, so that U pairs of dependent reads are in flight
-// together. A key whose first candidate is not it (another key with the same
-// tag, or a key stored past its home bucket) takes the full probe_one.
-template <int W, int U>
-__device__ __forceinline__ void probe_many(const uint8_t* __restrict__ tags, const uint64_t* __restrict__ table,
-                                           uint64_t n_buckets, const bool (&act)[U], const uint64_t (&h)[U],
-                                           uint64_t (&M)[U][W]) {
+// As mbar_try_wait, suspended for up to `ns` (a hint) before it answers no: a
+// warp that asks again and again takes issue slots from the chain warps.
+__device__ __forceinline__ bool mbar_try_wait_for(uint32_t mbar, uint32_t parity, uint32_t ns) {
+  uint32_t done;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
+      " selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(done) : "r"(mbar), "r"(parity), "r"(ns) : "memory");
+  return done != 0;
+}
+
+// A warp's bounded wait for a phase; false when it gave up, or when another warp of the
+// CTA did (*failed), after which every wait of the CTA ends at once.
+__device__ __forceinline__ bool mbar_wait_or(uint32_t mbar, uint32_t parity, volatile int* failed) {
+  bool ok = false;
+  for (uint32_t i = 0; i < kSpinLimit; ++i) {
+    ok = mbar_try_wait_for(mbar, parity, 4000);
+    if (ok || ((i & 15) == 15 && *failed)) break;
+  }
+  ok = __all_sync(kFull, ok);  // the warp goes on together
+  if (!ok) *failed = 1;
+  return ok;
+}
+
+// Eight chain steps: digests c in, hashes to o (which may be where c came from).
+template <bool EXACT>
+__device__ __forceinline__ uint64_t chain8(uint64_t h, const ulonglong2 (&c)[4], ulonglong2* o) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint64_t x = EXACT ? chain_step(h, c[i].x) : chain_raw(h, c[i].x);
+    h = EXACT ? chain_step(x, c[i].y) : chain_raw(x, c[i].y);
+    o[i] = make_ulonglong2(x, h);
+  }
+  return h;
+}
+
+__device__ __forceinline__ void load8(ulonglong2 (&c)[4], const ulonglong2* p) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) c[i] = p[i];
+}
+
+// Tier masks of a warp's keys, one per lane: the home-bucket tags, then the
+// tag matches' entries in turn for the whole warp (the first is the key's own
+// for all but ~4 % of the keys held), then probe_one for a key not in its
+// home bucket where that has keys stored past it.
+template <int W>
+__device__ __forceinline__ void probe_warp(const uint8_t* __restrict__ tags, const uint64_t* __restrict__ table,
+                                           uint64_t n_buckets, bool act, uint64_t h, uint64_t (&M)[W]) {
   constexpr int EW = entry_words(W);
   constexpr int NV = (W + 2) / 2;
-  uint64_t bk[U];
-  uint4 tv[U];
+  const uint64_t bk = home_bucket(h, n_buckets);
+  uint4 tv = make_uint4(0, 0, 0, 0);
+  if (act) tv = __ldg(reinterpret_cast<const uint4*>(tags + bk * kBucket));
+  uint32_t cand = act ? slot_match(tv, key_tag(h)) : 0;
+  bool found = false;
 #pragma unroll
-  for (int u = 0; u < U; ++u) {
-    bk[u] = act[u] ? home_bucket(h[u], n_buckets) : 0;
-    if (act[u]) tv[u] = __ldg(reinterpret_cast<const uint4*>(tags + bk[u] * kBucket));
-  }
-  ulonglong2 v[U][NV];
-  uint32_t cand[U];
+  for (int w = 0; w < W; ++w) M[w] = 0;
+  while (__any_sync(kFull, cand != 0)) {
+    if (cand) {
+      const ulonglong2* e = reinterpret_cast<const ulonglong2*>(table + (bk * kSlots + next_slot(cand)) * EW);
+      ulonglong2 v[NV];
 #pragma unroll
-  for (int u = 0; u < U; ++u) {
-    cand[u] = act[u] ? slot_match(tv[u], key_tag(h[u])) : 0;
-    if (cand[u]) {
-      const ulonglong2* e = reinterpret_cast<const ulonglong2*>(table + (bk[u] * kSlots + __ffs(cand[u]) - 1) * EW);
+      for (int q = 0; q < NV; ++q) v[q] = __ldg(e + q);
+      if (v[0].x == h) {
 #pragma unroll
-      for (int q = 0; q < NV; ++q) v[u][q] = __ldg(e + q);
+        for (int w = 0; w < W; ++w) M[w] = (w & 1) ? v[(w + 1) >> 1].x : v[(w + 1) >> 1].y;
+        found = true;
+        cand = 0;
+      }
     }
   }
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-#pragma unroll
-    for (int w = 0; w < W; ++w) M[u][w] = 0;
-    if (!act[u]) continue;
-    if (cand[u] && v[u][0].x == h[u]) {
-#pragma unroll
-      for (int w = 0; w < W; ++w) M[u][w] = (w & 1) ? v[u][(w + 1) >> 1].x : v[u][(w + 1) >> 1].y;
-    } else if ((cand[u] & (cand[u] - 1)) || overflow_count(tv[u])) {
-      probe_one<W>(tags, table, n_buckets, h[u], M[u]);  // more candidates, or later buckets
-    }
-    // else: no candidate left and no key stored past the home bucket: absent
-  }
+  if (act && !found && overflow_count(tv) != 0) probe_one<W>(tags, table, n_buckets, h, M);
+  __syncwarp();
 }
 
-// One thread per request: 1 if the request leads its group (the group
-// table's lowest request with its first-block hash), else 0.
+// The group stage, a warp per request: its leader (the lowest request with the
+// same first block, from the group table), the shared prefix (leading blocks
+// with the leader's digests) and whether the chain kernel takes the request.
+// With `defer`, a member with a short tail past its shared prefix is left to
+// the walk kernel, which chains only the tail, from the leader's hash: the
+// chain kernel then has the leaders and a few others.
+constexpr int kDeferTail = 256;  // blocks; the walk's steps take ~100 cycles each
+// The line: with four or fewer requests an SM nothing is deferred; with more, a
+// tail of a quarter of the prompt at most. 8,192 requests of the burst trace:
+// k_lead 14 us instead of 4, the chain kernel 99 instead of 165 (all requests
+// chained there), the walk 18.5 instead of 15.7.
+__device__ __forceinline__ bool short_tail(int64_t nb, int64_t sh) {
+  return nb - sh <= kDeferTail && 4 * (nb - sh) <= nb;
+}
+
 __global__ void __launch_bounds__(256)
     k_lead(const int64_t* __restrict__ block_off, int32_t n, const int32_t* __restrict__ batch_ok,
            const uint64_t* __restrict__ D, uint64_t h_init, const uint64_t* __restrict__ groups, uint64_t gmask,
-           uint8_t* __restrict__ lead_flag) {
+           bool defer, int32_t* __restrict__ lead, int32_t* __restrict__ share, uint8_t* __restrict__ active) {
   pdl_enter();
-  const int32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+  const int32_t r = (int32_t)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
+  const int lane = threadIdx.x & 31;
   if (r >= n || !*batch_ok) return;
-  const int64_t bo = block_off[r];
-  uint8_t f = 0;
-  if (block_off[r + 1] > bo) {
-    const uint64_t key = first_hash(h_init, __ldg(D + bo));
-    uint64_t sl = key & gmask;
-    for (uint64_t t = 0; t <= gmask; ++t, sl = (sl + 1) & gmask) {
-      const ulonglong2 pr = *reinterpret_cast<const ulonglong2*>(groups + 2 * sl);
-      if (pr.x == key) {
-        f = INT32_MAX - (int32_t)pr.y == r;
+  const int64_t bo = __ldg(block_off + r), nb = __ldg(block_off + r + 1) - bo;
+  int32_t l = r;
+  int64_t sh = 0;
+  if (nb > 0) {
+    const uint64_t key = chain_step(h_init, __ldg(D + bo));
+    const uint64_t s0 = key & gmask;
+    for (uint64_t t = 0; t <= gmask; t += 32) {
+      const uint64_t sl = (s0 + t + lane) & gmask;
+      const ulonglong2 e = *reinterpret_cast<const ulonglong2*>(groups + 2 * sl);
+      const unsigned hit = __ballot_sync(kFull, e.x == key), stop = hit | __ballot_sync(kFull, e.x == 0);
+      if (stop) {
+        const int first = __ffs(stop) - 1;
+        const int32_t who = __shfl_sync(kFull, INT32_MAX - (int32_t)e.y, first);
+        if (hit & (1u << first)) l = who;
         break;
       }
-      if (pr.x == 0) break;
+    }
+    if (l != r && l >= 0 && l < n) {
+      const int64_t lo = __ldg(block_off + l), nl = __ldg(block_off + l + 1) - lo;
+      const int64_t m = nb < nl ? nb : nl;
+      sh = m;
+      for (int64_t b = 0; b < m; b += 32 * kGroupAhead) {
+        bool ne[kGroupAhead];
+#pragma unroll
+        for (int u = 0; u < kGroupAhead; ++u) {
+          const int64_t bb = b + 32 * u + lane;
+          ne[u] = bb < m && __ldg(D + bo + bb) != __ldg(D + lo + bb);
+        }
+        int64_t first = -1;
+#pragma unroll
+        for (int u = 0; u < kGroupAhead; ++u) {
+          const unsigned x = __ballot_sync(kFull, ne[u]);
+          if (x && first < 0) first = 32 * u + __ffs(x) - 1;
+        }
+        if (first >= 0) {
+          sh = b + first;
+          break;
+        }
+      }
+    } else {
+      l = r;
     }
   }
-  lead_flag[r] = f;
+  if (lane == 0) {
+    lead[r] = l;
+    share[r] = (int32_t)sh;
+    active[r] = !(defer && sh > 0 && short_tail(nb, sh));
+  }
 }
 
+struct ChainArgs {
+  const int64_t* block_off;
+  const int64_t* chunk_off;
+  int32_t n;
+  int S;
+  uint64_t h_init;
+  const int32_t* batch_ok;
+  const uint64_t* D;
+  uint64_t* hashes;  // NULL: nobody reads them
+  uint64_t* sk_out;
+  const int32_t* share;    // leading blocks whose masks the walk reads from the group leader
+  const uint8_t* active;   // requests the kernel takes (the walk kernel chains the others' tails)
+  const uint8_t* tags;
+  const uint64_t* table;
+  uint64_t n_buckets;
+  uint64_t* masks;
+  uint64_t* chunk_and;
+  int32_t* status;
+  int deal;  // requests dealt by `active`
+  int chain_warps;
+  int slots;  // per lane of the ring, a power of two
+};
+
+// One chain warp's part of a round: its 32 lanes' streams, slot after slot, in
+// place: 32 digests become 32 hashes. The eight digests after those in work
+// are always loaded ahead, across slots too: whether the next slot is full is
+// asked eight steps before its first digests are loaded (slots are filled well
+// ahead, so the answer is nearly always yes; else the warp waits). The
+// sentinel remap of hashes 0 and 1 is left out unless
+// EXACT (~15 cycles a step): the probe warps look at every hash anyway, and
+// a round in which one is below 2 (once in 2^63 blocks) runs again, exactly.
+template <bool EXACT>
+__device__ __forceinline__ void chain_lanes(const ChainArgs& a, unsigned char* ring, const int32_t* s_at,
+                                            uint64_t* s_full, uint64_t* s_ready, int32_t* s_pos, int32_t len, int32_t m,
+                                            int* failed) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, lanes = 32 * a.chain_warps;
+  const int smask = a.slots - 1, sshift = 31 - __clz(a.slots);
+  const int32_t j = 32 * warp + lane;
+  unsigned char* const mine = ring + (size_t)j * kCpRow;
+  const uint32_t full = smem_u32(s_full + warp * kCpMaxSlots), ready = smem_u32(s_ready + warp * kCpMaxSlots);
+  if (len == 0) return;
+  int32_t i = j;                               // the stream's next request,
+  int32_t next = i < m ? s_at[i] : INT32_MAX;  // and the position where it begins
+  uint64_t h = a.h_init;
+  ulonglong2 c[4], x[4];
+  if (!mbar_wait_or(full, 0, failed)) {
+    if (lane == 0) latch_error(a.status, SMETRIC_ERR_CUDA);
+    return;
+  }
+  ulonglong2* row = reinterpret_cast<ulonglong2*>(mine);
+  load8(c, row);
+  for (int32_t q = 0; q < len; ++q) {
+    while (q == next) {  // (an empty request begins where the next one does)
+      h = a.h_init;
+      i += lanes;
+      next = i < m ? s_at[i] : INT32_MAX;
+    }
+    load8(x, row + 4);
+    h = chain8<EXACT>(h, c, row);
+    load8(c, row + 8);
+    h = chain8<EXACT>(h, x, row + 4);
+    const int32_t qn = q + 1 < len ? q + 1 : q;
+    const uint32_t bar = full + 8u * (uint32_t)(qn & smask), par = (uint32_t)(qn >> sshift) & 1u;
+    ulonglong2* const next_row = reinterpret_cast<ulonglong2*>(mine + (size_t)((qn & smask) * lanes) * kCpRow);
+    const bool there = mbar_try_wait(bar, par);
+    load8(x, row + 12);
+    h = chain8<EXACT>(h, c, row + 8);
+    // (the loads come after the answer: nothing else holds them back)
+    if (!__all_sync(kFull, there) && !mbar_wait_or(bar, par, failed)) {
+      if (lane == 0) latch_error(a.status, SMETRIC_ERR_CUDA);
+      return;
+    }
+    load8(c, next_row);
+    h = chain8<EXACT>(h, x, row + 12);
+    __syncwarp();
+    if (lane == 0) {
+      mbar_arrive(ready + 8u * (uint32_t)(q & smask));
+      *reinterpret_cast<volatile int32_t*>(s_pos + warp) = q + 1;
+    }
+    row = next_row;
+  }
+}
+
+struct __align__(16) ChainReq {
+  int64_t bo;     // first block in the batch
+  int64_t cb;     // first request-aligned chunk
+  int32_t nb;     // full blocks
+  int32_t share;  // leading blocks whose masks the group leader's probes give
+  int32_t req;
+};
+
+// W = 0: chain only (no index): hashes and session keys.
 template <int W>
-__global__ void __launch_bounds__(kCpWarps * 32, 1)
-    k_chain_probe(const int64_t* __restrict__ block_off, const int64_t* __restrict__ chunk_off, int32_t n, int S,
-                  uint64_t h_init, const int32_t* __restrict__ batch_ok, const uint64_t* __restrict__ D,
-                  uint64_t* __restrict__ hashes, uint64_t* __restrict__ sk_out, const uint64_t* __restrict__ groups,
-                  uint64_t gmask, int32_t* __restrict__ lead, int32_t* __restrict__ share,
-                  const uint8_t* __restrict__ tags,
-                  const uint64_t* __restrict__ table, uint64_t n_buckets, uint64_t* __restrict__ masks,
-                  uint64_t* __restrict__ chunk_and, const uint8_t* __restrict__ lead_flag, int chain_warps,
-                  int32_t* status) {
-  pdl_enter();
-  extern __shared__ __align__(128) unsigned char csm[];  // chain lanes' digest rings
-  __shared__ int32_t s_ready[kCpMaxGroup];  // chunks chained, per request of the group
-  __shared__ int32_t s_share[kCpMaxGroup];  // shared prefix per request (-1 until known)
-  __shared__ int32_t s_dead[kCpMaxGroup];   // first chunk whose AND is empty (INT32_MAX until one is)
-  __shared__ int32_t s_fin[kCpMaxGroup];    // chunks finished in order from the first unshared one
-  __shared__ int64_t s_bo[kCpMaxGroup];     // per request of the group: first block in the batch,
-  __shared__ int64_t s_cb[kCpMaxGroup];     // first request-aligned chunk,
-  __shared__ int32_t s_nb[kCpMaxGroup];     // and full blocks
-  __shared__ int32_t s_next0;               // work counter: share tasks
-  __shared__ unsigned long long s_next1;    // work counter: probe items
-  __shared__ int32_t s_maxch;               // most chunks of a request in the group
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // The CTAs' requests. A group leader (the lowest request with its first
-  // block, which probes its whole prefix) costs a member (which probes only
-  // past its shared prefix) many times over, so leaders are dealt round robin
-  // over the CTAs in request order, then the members after them: every CTA
-  // gets its share of each. k_lead has marked the leaders. Past 32 requests
-  // a thread, or kCpDealMax a CTA, requests are taken as blockIdx.x +
-  // k * gridDim.x instead.
-  __shared__ int32_t s_mine[kCpDealMax];
+__global__ void __launch_bounds__(cp_warps(W) * 32, 1) k_chain_probe(const ChainArgs a) {
+  extern __shared__ __align__(128) unsigned char csm[];  // the ring: slot s of lane j at (s * lanes + j) * kCpRow
+  // per request of the round, in lane order (request k of a round is the
+  // k / lanes-th of a lane's stream)
+  __shared__ ChainReq s_rq[kCpRound];
+  __shared__ int32_t s_at[kCpRound];    // first position in the lane's stream
+  __shared__ int32_t s_dead[kCpRound];  // first chunk whose AND is empty (INT32_MAX until one is)
+  __shared__ int32_t s_mine[kCpRound];
+  __shared__ int32_t s_len0[kCpRound];  // full blocks, in the order taken
+  __shared__ int32_t s_len[kCpMaxLanes];  // positions of each lane's stream
+  __shared__ int32_t s_most[kCpMaxChainWarps];  // and the most of a chain warp's lanes
+  __shared__ int32_t s_pos[kCpMaxChainWarps];   // positions each chain warp has chained
   __shared__ int32_t s_nmine;
   __shared__ int32_t s_wsum[kCpWarps];
-  const int32_t stride = (int32_t)gridDim.x;
+  __shared__ int s_failed;
+  __shared__ int s_redo;  // this round has met a hash below 2
+  __shared__ __align__(8) uint64_t s_full[kCpMaxChainWarps * kCpMaxSlots];
+  __shared__ __align__(8) uint64_t s_ready[kCpMaxChainWarps * kCpMaxSlots];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int32_t stride = (int32_t)gridDim.x, n = a.n;
+  const int lanes = 32 * a.chain_warps;
+  const int smask = a.slots - 1;
+  const int sshift = 31 - __clz(a.slots);
+  pdl_enter();
+  if (!*a.batch_ok) {
+    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)stride * blockDim.x)
+      a.sk_out[r] = 0;
+    return;
+  }
+  // The CTAs' requests: those k_lead left to this kernel are dealt round robin
+  // in request order, so that every CTA gets its share of them. Past 32
+  // requests a thread, or kCpRound a CTA (no request is left to the walk then),
+  // requests are taken as blockIdx.x + k * gridDim.x.
   const int32_t per_t = (n + (int32_t)blockDim.x - 1) / (int32_t)blockDim.x;
-  const bool dealt = *batch_ok && per_t <= 32 && (n + stride - 1) / stride <= kCpDealMax;
+  const bool dealt = W > 0 && a.deal;
   if (dealt) {
     if (threadIdx.x == 0) s_nmine = 0;
-    const int32_t a = min(n, (int32_t)threadIdx.x * per_t), e = min(n, a + per_t);
-    uint32_t lead_bits = 0;  // bit i: request a + i leads its group (from k_lead)
-    for (int32_t r = a; r < e; ++r) lead_bits |= (uint32_t)__ldg(lead_flag + r) << (r - a);
-    // exclusive scan of the leader counts over the threads, in request order
-    const int32_t cnt = __popc(lead_bits);
+    const int32_t lo = min(n, (int32_t)threadIdx.x * per_t), hi = min(n, lo + per_t);
+    uint32_t bits = 0;  // bit i: request lo + i is this kernel's
+    for (int32_t r = lo; r < hi; ++r) bits |= (uint32_t)__ldg(a.active + r) << (r - lo);
+    // exclusive scan of the counts over the threads, in request order
+    const int32_t cnt = __popc(bits);
     int32_t incl = cnt;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -903,268 +1011,179 @@ __global__ void __launch_bounds__(kCpWarps * 32, 1)
     }
     if (lane == 31) s_wsum[warp] = incl;
     __syncthreads();
-    int32_t before = 0, total = 0;
-    for (int w2 = 0; w2 < kCpWarps; ++w2) {
-      const int32_t v = s_wsum[w2];
-      if (w2 < warp) before += v;
-      total += v;
-    }
-    int32_t lrank = before + incl - cnt;  // leaders before request a
-    for (int32_t r = a; r < e; ++r) {
-      const bool isl = (lead_bits >> (r - a)) & 1u;
-      // leaders by leader rank; members by member rank, continuing the deal
-      const int32_t cta = isl ? lrank % stride : (total + (r - lrank)) % stride;
-      if (isl) ++lrank;
-      if (cta == (int32_t)blockIdx.x) s_mine[atomicAdd(&s_nmine, 1)] = r;
-    }
+    int32_t rank = incl - cnt;
+    for (int w2 = 0; w2 < warp; ++w2) rank += s_wsum[w2];
+    for (; bits; bits &= bits - 1, ++rank)
+      if (rank % stride == (int32_t)blockIdx.x) s_mine[atomicAdd(&s_nmine, 1)] = lo + __ffs(bits) - 1;
     __syncthreads();
   }
-  const int32_t m = dealt ? s_nmine : n > (int32_t)blockIdx.x ? (n - (int32_t)blockIdx.x + stride - 1) / stride : 0;
-  auto req_of = [&](int32_t k) { return dealt ? s_mine[k] : (int32_t)blockIdx.x + k * stride; };
-  if (!*batch_ok) {
-    for (int32_t k = (int32_t)threadIdx.x; k < m; k += blockDim.x) sk_out[req_of(k)] = 0;
-    return;
-  }
-  // chain warps: warp k on scheduler k (one each); every other warp probes
-  const int cw = warp;
-  const bool chain = warp < chain_warps;
-  const bool prober = warp >= chain_warps;
-  const int G = 32 * chain_warps;
+  const int32_t m_all = dealt ? s_nmine
+                              : n > (int32_t)blockIdx.x ? (n - (int32_t)blockIdx.x + stride - 1) / stride : 0;
 
-  for (int32_t g0 = 0; g0 < m; g0 += G) {
-    const int mg = min(G, m - g0);
-    if ((int)threadIdx.x < mg) {
-      s_ready[threadIdx.x] = 0;
-      s_share[threadIdx.x] = -1;
-      s_dead[threadIdx.x] = INT32_MAX;
-      s_fin[threadIdx.x] = 0;
-      const int32_t r = req_of(g0 + (int32_t)threadIdx.x);
-      const int64_t bo = block_off[r];
-      s_bo[threadIdx.x] = bo;
-      s_nb[threadIdx.x] = (int32_t)(block_off[r + 1] - bo);
-      s_cb[threadIdx.x] = chunk_off[r];
+  bool again = false, used = false;  // the round before met a sentinel; barriers exist
+  for (int32_t g0 = 0; g0 < m_all; g0 += again ? 0 : kCpRound) {
+    const int32_t m = min(kCpRound, m_all - g0);
+    const int act = min(m, lanes);  // lanes in use
+    // ---- the round's requests; with more than one per lane, longest first
+    int32_t k = -1, r = 0, nb = 0;  // this thread's request: its place in lane order, index and full blocks
+    if (threadIdx.x < (unsigned)m) {
+      k = (int32_t)threadIdx.x;
+      r = dealt ? s_mine[g0 + k] : (int32_t)blockIdx.x + (g0 + k) * stride;
+      nb = (int32_t)(__ldg(a.block_off + r + 1) - __ldg(a.block_off + r));
+      s_len0[k] = nb;
     }
+    if (threadIdx.x < kCpMaxLanes) s_len[threadIdx.x] = 0;
+    if (threadIdx.x < kCpMaxChainWarps) s_most[threadIdx.x] = s_pos[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
-      s_next0 = 0;
-      s_next1 = 0;
-      s_maxch = 0;
+      s_failed = 0;
+      s_redo = again;
+      for (int i = 0; i < a.chain_warps; ++i) {
+        const int in_use = min(32, act - 32 * i);
+        for (int s = 0; s < a.slots; ++s) {
+          if (used) {
+            asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(smem_u32(s_full + i * kCpMaxSlots + s)) : "memory");
+            asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(smem_u32(s_ready + i * kCpMaxSlots + s)) : "memory");
+          }
+          mbar_init(smem_u32(s_full + i * kCpMaxSlots + s), (uint32_t)max(1, in_use));
+          mbar_init(smem_u32(s_ready + i * kCpMaxSlots + s), 1);
+        }
+      }
     }
     __syncthreads();
-    if ((int)threadIdx.x < mg)
-      atomicMax(&s_maxch, (int32_t)(chunk_off[req_of(g0 + threadIdx.x) + 1] - chunk_off[req_of(g0 + threadIdx.x)]));
+    if (k >= 0) {
+      if (m > lanes) {  // by length, each pass over the lanes against the last: long after short
+        int32_t rank = 0;
+        for (int32_t i = 0; i < m; ++i) {
+          const int32_t v = s_len0[i];
+          rank += v > nb || (v == nb && i < (int32_t)threadIdx.x);
+        }
+        const int32_t pass = rank / lanes, at = rank % lanes;
+        k = pass * lanes + ((pass & 1) ? at : min(lanes, m - pass * lanes) - 1 - at);
+      }
+    }
     __syncthreads();
-    const int32_t maxch = s_maxch;
-    if (chain) {
-      // lane = request j of the group: the chain over its digests, one chunk
-      // at a time from a two-slot ring in shared memory (slot q & 1 holds
-      // chunk q; chunk q + 1 is copied in while chunk q is chained)
-      const int j = 32 * cw + lane;
-      const bool act = j < mg;
-      const int32_t r = act ? req_of(g0 + j) : 0;
-      int64_t bo = 0, nb = 0;
-      if (act) {
-        bo = __ldg(block_off + r);
-        nb = __ldg(block_off + r + 1) - bo;
+    if (k >= 0) {
+      ChainReq x = {};
+      x.bo = __ldg(a.block_off + r);
+      x.nb = nb;
+      x.req = r;
+      if (W > 0) {
+        x.cb = __ldg(a.chunk_off + r);
+        x.share = __ldg(a.share + r);
+        s_dead[k] = INT32_MAX;
       }
-      const int32_t nch = (int32_t)((nb + kChunk - 1) / kChunk);
-      int32_t wmax = nch;
-#pragma unroll
-      for (int dd = 16; dd > 0; dd >>= 1) wmax = max(wmax, __shfl_xor_sync(kFull, wmax, dd));
-      unsigned char* const ring = csm + (size_t)j * kCpRingBytes;
-      const uint32_t ring_s = smem_u32(ring);
-      // copies chunk q's digests [first, first + nv) in 16-byte pieces from the
-      // even index at or below first into slot q & 1
-      auto fetch = [&](int32_t q) {
-        const int64_t first = bo + (int64_t)kChunk * q;
-        const int64_t a = first & ~(int64_t)1;
-        const int nv = (int)min((int64_t)kChunk, nb - (int64_t)kChunk * q);
-        const int pieces = (int)((first + nv - a + 1) >> 1);
-        const uint32_t dst = ring_s + (uint32_t)((q & 1) * kCpRingDigests * 8);
-        for (int i = 0; i < pieces; ++i) cp_async16(dst + 16u * i, D + a + 2 * i);
-      };
-      if (act && nch > 0) fetch(0);
-      cp_async_commit();
-      uint64_t h = h_init;
-      for (int32_t q = 0; q < wmax; ++q) {
-        cp_async_wait_all();
-        if (q + 1 < nch) fetch(q + 1);
-        cp_async_commit();
-        if (q < nch) {
-          const int64_t b0 = (int64_t)kChunk * q;
-          const int nv = (int)min((int64_t)kChunk, nb - b0);
-          const uint64_t* dsm =
-              reinterpret_cast<const uint64_t*>(ring + (q & 1) * kCpRingDigests * 8) + ((bo + b0) & 1);
-          uint64_t* const ho = hashes + bo + b0;
-          for (int i = 0; i < nv; ++i) {
-            h = chain_step(h, dsm[i]);
-            ho[i] = h;
-          }
-          __threadfence_block();
-          st_release_cta(&s_ready[j], q + 1);  // the chunk's hashes are out
-        }
+      s_rq[k] = x;
+      if (nb == 0) a.sk_out[r] = 0;
+    }
+    __syncthreads();
+    if (threadIdx.x < (unsigned)act) {
+      int32_t pos = 0;
+      for (int32_t i = (int32_t)threadIdx.x; i < m; i += lanes) {
+        s_at[i] = pos;
+        pos += (s_rq[i].nb + kChunk - 1) / kChunk;
       }
-      cp_async_wait_all();
-      if (act) sk_out[r] = nb > 0 ? hashes[bo + (nb < S ? nb : (int64_t)S) - 1] : 0;
-    } else if (prober) {
-      // Phase 1, a warp per request (taken from a counter): the group leader
-      // (lowest request id with the same first-block hash, from the table the
-      // digest kernel filled) and the number of leading blocks whose digests
-      // equal the leader's.
-      for (;;) {
-        int32_t j = 0;
-        if (lane == 0) j = atomicAdd(&s_next0, 1);
-        j = __shfl_sync(kFull, j, 0);
-        if (j >= mg) break;
-        const int32_t r = req_of(g0 + j);
-        const int64_t bo = __ldg(block_off + r), nb = __ldg(block_off + r + 1) - bo;
-        int32_t l = r;
-        int64_t sh = 0;
-        if (nb > 0) {
-          const uint64_t key = first_hash(h_init, __ldg(D + bo));
-          const uint64_t s0 = key & gmask;
-          for (uint64_t t = 0; t <= gmask; t += 32) {
-            const uint64_t sl = (s0 + t + lane) & gmask;
-            const uint64_t k = groups[2 * sl];
-            const unsigned hit = __ballot_sync(kFull, k == key), emp = __ballot_sync(kFull, k == 0);
-            const unsigned stop = hit | emp;
-            if (stop) {
-              const int first = __ffs(stop) - 1;
-              if (hit & (1u << first)) l = INT32_MAX - (int32_t)groups[2 * ((s0 + t + first) & gmask) + 1];
-              break;
-            }
-          }
-          if (l != r && l >= 0 && l < n) {
-            const int64_t lo = __ldg(block_off + l), nl = __ldg(block_off + l + 1) - lo;
-            const int64_t m = nb < nl ? nb : nl;
-            sh = m;
-            for (int64_t b = 0; b < m; b += 32 * kGroupAhead) {
-              bool ne[kGroupAhead];
-#pragma unroll
-              for (int u = 0; u < kGroupAhead; ++u) {
-                const int64_t bb = b + 32 * u + lane;
-                ne[u] = bb < m && __ldg(D + bo + bb) != __ldg(D + lo + bb);
-              }
-              int64_t first = -1;
-#pragma unroll
-              for (int u = 0; u < kGroupAhead; ++u) {
-                const unsigned x = __ballot_sync(kFull, ne[u]);
-                if (x && first < 0) first = 32 * u + __ffs(x) - 1;
-              }
-              if (first >= 0) {
-                sh = b + first;
-                break;
-              }
-            }
-          } else {
-            l = r;
-          }
-        }
-        if (lane == 0) {
-          lead[r] = l;
-          share[r] = (int32_t)sh;
-          st_release_cta(&s_share[j], (int32_t)sh);
-        }
+      s_len[threadIdx.x] = pos;
+      atomicMax(&s_most[threadIdx.x >> 5], pos);
+    }
+    if (threadIdx.x == 0) asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    __syncthreads();
+    int32_t most = 0;
+    for (int i = 0; i < a.chain_warps; ++i) most = max(most, s_most[i]);
+
+    // The request of lane j's stream at position q (q < s_len[j]).
+    auto find = [&](int32_t q, int32_t j) {
+      int32_t i = j;
+      while (i + lanes < m && s_at[i + lanes] <= q) i += lanes;
+      return i;
+    };
+    auto row_of = [&](int32_t q, int32_t j) {
+      return reinterpret_cast<uint64_t*>(csm + (size_t)((q & smask) * lanes + j) * kCpRow);
+    };
+    // Position q of lane j: this lane's stored digest (0 past the request's end).
+    auto fill_load = [&](int32_t q, int32_t j) -> uint64_t {
+      if (q >= s_len[j]) return 0;
+      const int32_t i = find(q, j), b = kChunk * (q - s_at[i]) + lane;
+      return b < s_rq[i].nb ? __ldg(a.D + s_rq[i].bo + b) : 0;
+    };
+    auto fill_store = [&](int32_t q, int32_t j, uint64_t d) {
+      row_of(q, j)[lane] = d;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(s_full + (j >> 5) * kCpMaxSlots + (q & smask)));
+    };
+
+    if (warp < a.chain_warps) {
+      if (!s_redo)
+        chain_lanes<false>(a, csm, s_at, s_full, s_ready, s_pos, s_most[warp], m, &s_failed);
+      else
+        chain_lanes<true>(a, csm, s_at, s_full, s_ready, s_pos, s_most[warp], m, &s_failed);
+    } else {
+      // the first positions of every lane
+      const int pw = warp - a.chain_warps, npw = cp_warps(W) - a.chain_warps;
+      for (int32_t t = pw; t < act * a.slots; t += npw) {
+        const int32_t q = t / act, j = t - q * act;
+        if (q >= s_most[j >> 5]) continue;
+        fill_store(q, j, fill_load(q, j));
       }
-      // Phase 2: items (q, j) in chunk-major order, kCpProbes at a time: the
-      // tier masks of chunk q's blocks of request j at or past its shared
-      // prefix, once its chain has published the chunk; and the chunk's AND
-      // (a block not probed counts as all ones). Skipped with no wait: a chunk
-      // wholly inside the shared prefix (the walk reads the leader's). Skipped
-      // after waiting: any chunk after one whose AND is empty (that chunk
-      // lacks a block of every tier, so every run has ended there: the walk
-      // stops before reaching later chunks). When the probers' items in
-      // flight would span more than two rounds of the group (few requests per
-      // CTA), a request's chunk q starts only once its chunk q - 2 has
-      // finished (chunks then finish in order), so at most two of its chunks
-      // are probed ahead of knowing whether its runs are over.
-      const bool paced = (kCpWarps - chain_warps) * kCpProbes > 2 * mg;
-      const int64_t items = (int64_t)maxch * mg;
-      for (;;) {
-        int64_t t0 = 0;
-        if (lane == 0) t0 = (int64_t)atomicAdd(&s_next1, (unsigned long long)kCpProbes);
-        t0 = __shfl_sync(kFull, t0, 0);
-        if (t0 >= items) break;
-        // item t is chunk t / mg of request t % mg; one division per grab
-        int32_t q0 = (int32_t)(t0 < INT32_MAX ? (uint32_t)t0 / (uint32_t)mg : t0 / mg);
-        int32_t j0 = (int32_t)(t0 - (int64_t)q0 * mg);
-        bool act[kCpProbes];
-        uint64_t hv[kCpProbes];
-        int64_t f[kCpProbes], cidx[kCpProbes];
-        int32_t qs[kCpProbes], js[kCpProbes], rel[kCpProbes];  // rel: chunk index counted from the first unshared one
-#pragma unroll
-        for (int u = 0; u < kCpProbes; ++u) {
-          act[u] = false;
-          hv[u] = 0;
-          f[u] = 0;
-          cidx[u] = -1;
-          rel[u] = -1;
-          const int64_t t = t0 + u;
-          const int32_t q = q0, j = j0;
-          if (++j0 == mg) {
-            j0 = 0;
-            ++q0;
-          }
-          if (t >= items) continue;
-          qs[u] = q;
-          js[u] = j;
-          const int64_t bo = s_bo[j], nb = s_nb[j];
-          if ((int64_t)kChunk * q >= nb) continue;  // the request has no chunk q
-          if (!wait_above(&s_share[j], -1)) {
-            if (lane == 0) latch_error(status, SMETRIC_ERR_CUDA);
-            continue;
-          }
-          const int64_t sh = s_share[j];
-          if ((int64_t)kChunk * (q + 1) <= sh) continue;
-          rel[u] = paced ? q - (int32_t)(sh / kChunk) : -1;
-          if (paced && !wait_above(&s_fin[j], rel[u] - 2)) {  // chunk q - 2 has finished
-            if (lane == 0) latch_error(status, SMETRIC_ERR_CUDA);
-            rel[u] = -1;
-            continue;
-          }
-          if (ld_acquire_cta(&s_dead[j]) < q) continue;  // finished as skipped below
-          if (!wait_above(&s_ready[j], q)) {
-            if (lane == 0) latch_error(status, SMETRIC_ERR_CUDA);
-            continue;
-          }
-          const int64_t b = (int64_t)kChunk * q + lane;
-          act[u] = b < nb && b >= sh;
-          f[u] = bo + b;
-          cidx[u] = s_cb[j] + q;
-          if (act[u]) hv[u] = ld_relaxed_cta(hashes + bo + b);
+      // items in position-major order, every npw-th one
+      const int32_t dq = npw / act, dj = npw - dq * act;
+      int32_t q = pw / act, j = pw - q * act;
+      for (; q < most; q += dq, j += dj) {
+        if (j >= act) {
+          j -= act;
+          if (++q >= most) break;
         }
-        uint64_t M[kCpProbes][W];
-        probe_many<W, kCpProbes>(tags, table, n_buckets, act, hv, M);
+        const int32_t cw = j >> 5;
+        if (q >= s_most[cw]) continue;
+        const bool refill = q + a.slots < s_most[cw];
+        const uint64_t d = refill ? fill_load(q + a.slots, j) : 0;
+        if ((q >= a.slots && !poll_at_least(s_pos + cw, q - a.slots + 1, &s_failed)) ||
+            !mbar_wait_or(smem_u32(s_ready + cw * kCpMaxSlots + (q & smask)), (q >> sshift) & 1, &s_failed)) {
+          if (lane == 0) latch_error(a.status, SMETRIC_ERR_CUDA);
+          break;
+        }
+        const uint64_t h = row_of(q, j)[lane];
+        __syncwarp();
+        if (refill) fill_store(q + a.slots, j, d);
+        if (q >= s_len[j]) continue;
+        const int32_t i = find(q, j);
+        const ChainReq x = s_rq[i];
+        const int32_t c = q - s_at[i], b = kChunk * c + lane;
+        const bool in = b < x.nb;
+        if (in) {
+          if (h < 2) s_redo = 1;
+          if (a.hashes) a.hashes[x.bo + b] = h;
+          if (b == min(x.nb, a.S) - 1) a.sk_out[x.req] = h;
+        }
+        if constexpr (W > 0) {
+          // nothing to probe in a chunk wholly inside the shared prefix (the walk reads the
+          // leader's), nor after one whose AND is empty (every run has ended there)
+          const int32_t dead = __shfl_sync(kFull, *(volatile int32_t*)&s_dead[i], 0);
+          if (kChunk * (c + 1) <= x.share || dead < c) continue;
+          const bool on = in && b >= x.share;
+          uint64_t M[W];
+          probe_warp<W>(a.tags, a.table, a.n_buckets, on, h, M);
+          if (on) {
+            uint64_t* const out = a.masks + (x.bo + b) * W;
 #pragma unroll
-        for (int u = 0; u < kCpProbes; ++u) {
-          if (cidx[u] < 0) continue;  // warp-uniform
-          if (act[u]) {
-#pragma unroll
-            for (int w = 0; w < W; ++w) masks[f[u] * W + w] = M[u][w];
+            for (int w = 0; w < W; ++w) out[w] = M[w];
           }
           bool empty = true;
 #pragma unroll
           for (int w = 0; w < W; ++w) {
-            const uint64_t x = act[u] ? M[u][w] : ~0ull;
-            const uint64_t a = (uint64_t)__reduce_and_sync(kFull, (unsigned)x) |
-                               ((uint64_t)__reduce_and_sync(kFull, (unsigned)(x >> 32)) << 32);
-            if (lane == w) chunk_and[cidx[u] * W + w] = a;
-            empty &= a == 0;
+            const uint64_t y = on ? M[w] : ~0ull;
+            const uint64_t v = (uint64_t)__reduce_and_sync(kFull, (unsigned)y) |
+                               ((uint64_t)__reduce_and_sync(kFull, (unsigned)(y >> 32)) << 32);
+            if (lane == w) a.chunk_and[(x.cb + c) * W + w] = v;
+            empty &= v == 0;
           }
-          if (empty && lane == 0) atomicMin(&s_dead[js[u]], qs[u]);
-        }
-        // chunks finish in order: after the request's previous chunk
-#pragma unroll
-        for (int u = 0; u < kCpProbes; ++u) {
-          if (rel[u] < 0) continue;  // warp-uniform
-          if (lane == 0) {
-            if (!wait_above(&s_fin[js[u]], rel[u] - 1)) latch_error(status, SMETRIC_ERR_CUDA);
-            st_release_cta(&s_fin[js[u]], rel[u] + 1);
-          }
-          __syncwarp();
+          if (empty && lane == 0) atomicMin(&s_dead[i], c);
         }
       }
     }
-    __syncthreads();  // the group's shared state is rewritten by the next group
+    __syncthreads();
+    used = true;
+    again = !again && s_redo && !s_failed;
+    __syncthreads();  // the round's shared state is rewritten by the next one
   }
 }
 
@@ -1174,6 +1193,7 @@ enum Decide { kArgmin = 0, kSession = 1, kColoc = 2, kBailian = 3, kLMetric = 4 
 
 struct WalkPolicy {
   int on;    // a Decide value; 0 = the argmin cost
+  int summ;  // also record every request's run ends (the sequential variant reads them)
   int64_t c_lin, c_att, d0, d1, hit_num, hit_den;
   int32_t rr_base;
   const int32_t* turn;
@@ -1184,46 +1204,71 @@ struct WalkPolicy {
   int64_t lam_num, lam_den;  // Bailian's weight
 };
 
+struct WalkArgs {
+  int N, B, S;
+  const int64_t* off;
+  const int64_t* block_off;
+  const int64_t* chunk_off;
+  int32_t n;
+  const int64_t* load;
+  int64_t w_load, w_miss, w_glob;
+  const uint64_t* masks;
+  const uint64_t* chunk_and;
+  const int32_t* batch_ok;
+  const int32_t* lead;
+  const int32_t* share;
+  int32_t* summ;
+  int32_t* inst_out;
+  int32_t* lhit_out;
+  int32_t* ghit_out;
+  uint4* groups;
+  int64_t group_vecs;
+  // k_lead's marks, when it left members' tails to this kernel (NULL: it did not)
+  const uint8_t* active;
+  const uint64_t* D;
+  uint64_t* hashes;
+  bool want_hashes;
+  uint64_t* sk_out;
+  const uint8_t* tags;
+  const uint64_t* table;
+  uint64_t n_buckets;
+};
+
 // One warp per request, lanes = 32 consecutive blocks. The masks are
 // AND-scanned across lanes; lane j's "death set" is the local tiers held
-// through block j-1 but not through block j. Lanes with a non-empty death set
-// append an event (block, set) to the warp's list in shared memory; a request
-// has at most one event per instance and usually two or three in all. The
+// through block j-1 but not through block j. A block where runs end (two or
+// three of a request's have any) hands its set to the lanes that hold those
+// instances: lane i keeps c of instances i, i + 32, ... in registers. The
 // global-tier run is the first lane whose block the global tier lacks. Then
-// lanes = instances: c_i = the block of the first event containing i (or n_r
-// if i held every block), the cost, and a shuffle argmin with ties to the
-// lowest id.
+// lanes = instances for the cost and a shuffle argmin with ties to the lowest id.
 //
-// One pass over every request. A member's blocks before `share` are its
-// leader's, whose masks and chunk ANDs the probe wrote (the member's own were
-// not probed there): its walk reads them from the leader up to block
-// `share` (a 32-block chunk that straddles `share` block by block), then its
-// own. Every request's run ends (c_i for every instance, then g) go to
-// `summ` for the sequential variant.
+// A member's blocks before `share` are its leader's, whose masks and chunk ANDs
+// the probe wrote (the member's own were not probed there): its walk reads them
+// from the leader up to block `share` (a 32-block chunk that straddles `share`
+// block by block), then its own.
+//
+// A member that k_lead did not leave to the chain kernel has only its shared
+// prefix there. Its tail past `share` is chained here as far as it is needed,
+// all lanes in step from the leader's hash: the first block alone, which ends
+// most walks (a tail is mostly a request's fresh tokens, which no tier holds),
+// then 32 blocks at a time.
 template <int W, int DECIDE>
-__global__ void __launch_bounds__(kMatchWarps * 32, 5)
-    k_walk(int N, int B, const int64_t* __restrict__ off, const int64_t* __restrict__ block_off, int32_t n,
-           const int64_t* __restrict__ load, int64_t w_load, int64_t w_miss, int64_t w_glob,
-           const uint64_t* __restrict__ masks, const uint64_t* __restrict__ chunk_and,
-           const int64_t* __restrict__ chunk_off, const int32_t* __restrict__ batch_ok,
-           const int32_t* __restrict__ lead, const int32_t* __restrict__ share, int32_t* __restrict__ summ,
-           int32_t* __restrict__ inst_out, int32_t* __restrict__ lhit_out,
-           int32_t* __restrict__ ghit_out, uint4* __restrict__ groups, int64_t group_vecs,
-           const WalkPolicy pol) {
+__global__ void __launch_bounds__(kMatchWarps * 32, 4) k_walk(const WalkArgs a, const WalkPolicy pol) {
   pdl_enter();
-  extern __shared__ int64_t msm[];
-  int64_t* load_s = msm;                                                     // [N]
+  const int N = a.N, B = a.B;
+  const int32_t n = a.n;
+  const int64_t w_load = a.w_load, w_miss = a.w_miss, w_glob = a.w_glob;
+  int32_t* const inst_out = a.inst_out;
+  int32_t* const lhit_out = a.lhit_out;
+  int32_t* const ghit_out = a.ghit_out;
+  __shared__ int64_t load_s[SMETRIC_MAX_INSTANCES];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // per warp: N events of (block, W mask words)
-  uint64_t* ev_mask = reinterpret_cast<uint64_t*>(msm + N) + (size_t)warp * N * W;
-  int64_t* ev_pos = msm + N + (size_t)kMatchWarps * N * W + (size_t)warp * N;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) load_s[i] = load[i];
+  for (int i = threadIdx.x; i < N; i += blockDim.x) load_s[i] = a.load[i];
   __syncthreads();
-  const bool ok = *batch_ok != 0;
+  const bool ok = *a.batch_ok != 0;
   const int gword = N >> 6;
   const uint64_t gbit = 1ull << (N & 63);
   const int64_t tw = (int64_t)gridDim.x * kMatchWarps;
-  const unsigned lt = (1u << lane) - 1;
 
   if (!ok)
     for (int64_t r = (int64_t)blockIdx.x * kMatchWarps + warp; r < n; r += tw)
@@ -1232,51 +1277,45 @@ __global__ void __launch_bounds__(kMatchWarps * 32, 5)
         if (DECIDE == kSession || DECIDE == kColoc) pol.stick[r] = 0;
       }
   for (int64_t r = (int64_t)blockIdx.x * kMatchWarps + warp; ok && r < n; r += tw) {
-    const int64_t L = off[r + 1] - off[r];
+    const int64_t L = a.off[r + 1] - a.off[r];
     const int64_t nb = L / B;
-    const int64_t bo = block_off[r];
-    const int64_t sh = share[r];  // 0 for a leader
-    const int32_t l = sh > 0 ? lead[r] : (int32_t)r;
+    const int64_t bo = a.block_off[r];
+    const int64_t sh = a.share[r];  // 0 for a leader
+    const int32_t l = sh > 0 ? a.lead[r] : (int32_t)r;
+    const bool tail = a.active && !a.active[r];
     // chunk ANDs are per request-aligned chunk: blocks 32q .. 32q + 31 of
     // request r at index chunk_off[r] + q; block p < sh of the request is
     // block p of its leader
-    const int64_t cbase = __ldg(chunk_off + r);
-    const int64_t lbo = sh > 0 ? __ldg(block_off + l) : bo;
-    const int64_t lcb = sh > 0 ? __ldg(chunk_off + l) : cbase;
-    auto mask_at = [&](int64_t p, int w) -> uint64_t {  // block p of the request
-      return __ldg(masks + ((p < sh ? lbo : bo) + p) * W + w);
+    const int64_t cbase = __ldg(a.chunk_off + r);
+    const int64_t lbo = sh > 0 ? __ldg(a.block_off + l) : bo;
+    const int64_t lcb = sh > 0 ? __ldg(a.chunk_off + l) : cbase;
+    // masks of the blocks from block p on, lane = block (all ones past `end`)
+    auto masks_at = [&](int64_t p, int64_t end, uint64_t (&x)[W]) {
+      const int64_t b = p + lane;
+      const uint64_t* const m = a.masks + ((b < sh ? lbo : bo) + b) * W;
+#pragma unroll
+      for (int w = 0; w < W; ++w) x[w] = b < end ? __ldg(m + w) : ~0ull;
     };
     auto and_at = [&](int64_t q, int w) -> uint64_t {  // its chunk q; 0 where the chunk straddles sh
-      if (32 * (q + 1) <= sh) return __ldg(chunk_and + (lcb + q) * W + w);
+      if (32 * (q + 1) <= sh) return __ldg(a.chunk_and + (lcb + q) * W + w);
       if (32 * q < sh) return 0ull;  // walked block by block
-      return __ldg(chunk_and + (cbase + q) * W + w);
+      return __ldg(a.chunk_and + (cbase + q) * W + w);
     };
-    int64_t f = bo;
-    const int64_t F1 = bo + nb;
-    const bool head_single = F1 - f < 32;
-    uint64_t pre[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-      if (head_single) {
-        const int64_t len = F1 - f;
-        pre[w] = lane < len ? mask_at(lane, w) : ~0ull;
-      } else {
-        pre[w] = lane < (nb >> 5) ? and_at(lane, w) : 0;
-      }
-    }
     constexpr int CT = 2 * W;  // groups of 32 covering the N + 1 <= 64 W tiers
-    uint64_t A[W];  // local tiers holding every block so far (warp-uniform)
+    int32_t c[CT];             // c of instance 32 t + lane
+    uint64_t A[W];             // local tiers holding every block so far (warp-uniform)
     bool galive = true;
     int64_t g = 0;
+#pragma unroll
+    for (int t = 0; t < CT; ++t) c[t] = (int32_t)nb;  // until its run ends
 #pragma unroll
     for (int w = 0; w < W; ++w) {
       const int lo = w * 64;
       A[w] = N >= lo + 64 ? ~0ull : (N > lo ? (1ull << (N - lo)) - 1 : 0ull);
     }
-    int ne = 0;
     // `len` consecutive blocks from request block `base`, lane j < len holding
-    // block base + j (lanes past len hold all ones): the runs that end there
-    // become events; returns true once no run is alive
+    // block base + j (lanes past len hold all ones): records the runs that end
+    // there; returns true once no run is alive
     auto span = [&](int64_t base, int len, const uint64_t (&x)[W]) -> bool {
       if (galive) {
         uint64_t mg = 0;
@@ -1303,59 +1342,77 @@ __global__ void __launch_bounds__(kMatchWarps * 32, 5)
         A[w] = __shfl_sync(kFull, v, 31);
         any |= A[w] != 0;
       }
-      const unsigned ev = __ballot_sync(kFull, dies);
-      if (dies) {
-        const int at = ne + __popc(ev & lt);
-        ev_pos[at] = base + lane;
+      for (unsigned ev = __ballot_sync(kFull, dies); ev; ev &= ev - 1) {
+        const int at = __ffs(ev) - 1;
 #pragma unroll
-        for (int w = 0; w < W; ++w) ev_mask[at * W + w] = X[w];
+        for (int w = 0; w < W; ++w) {
+          const uint64_t v = __shfl_sync(kFull, X[w], at);
+          if (((uint32_t)v >> lane) & 1u) c[2 * w] = (int32_t)base + at;
+          if (((uint32_t)(v >> 32) >> lane) & 1u) c[2 * w + 1] = (int32_t)base + at;
+        }
       }
-      ne += __popc(ev);
       return !any && !galive;
     };
-    bool dead = !galive;
-#pragma unroll
-    for (int w = 0; w < W; ++w) dead &= A[w] == 0;
-    // From block sh: single blocks up to a 32-aligned request position, then
     // 32 chunks per step from their AND summaries (lane = chunk); the first
-    // chunk that ends an alive run is walked block by block, and the request's
-    // last partial chunk too. The first step uses the loads issued above.
-    bool first = true;
-    while (!dead && f < F1) {
+    // chunk that ends an alive run is walked block by block, and the last
+    // partial chunk too (for a tail chained here: the shared prefix's).
+    const int64_t summed = tail ? sh : nb;  // blocks with masks and chunk ANDs
+    bool dead = false;
+    for (int64_t p = 0; !dead && p < summed;) {
       uint64_t x[W];
-      if (((f - bo) & 31) || F1 - f < 32) {
-        const int len = (int)min((int64_t)(32 - ((f - bo) & 31)), F1 - f);
+      const int64_t nfull = (summed - p) >> 5;
+      if (nfull > 0) {
 #pragma unroll
-        for (int w = 0; w < W; ++w)
-          x[w] = first ? pre[w] : lane < len ? mask_at(f - bo + lane, w) : ~0ull;
-        first = false;
-        dead = span(f - bo, len, x);
+        for (int w = 0; w < W; ++w) x[w] = lane < nfull ? and_at((p >> 5) + lane, w) : 0;
+        bool stop = lane >= nfull;
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+          stop |= (x[w] & A[w]) != A[w];
+          if (w == gword && galive) stop |= !(x[w] & gbit);
+        }
+        const unsigned sm = __ballot_sync(kFull, stop);
+        const int k = sm ? __ffs(sm) - 1 : 32;
+        p += 32 * (int64_t)k;  // chunks that keep every alive run
+        if (galive) g = p;
+        if (k >= nfull || k == 32) continue;
+      }
+      masks_at(p, summed, x);
+      dead = span(p, (int)min((int64_t)32, summed - p), x);
+      p += 32;
+    }
+    if (tail) {
+      const int64_t kS = min(nb, (int64_t)a.S) - 1;
+      uint64_t h = a.hashes[lbo + sh - 1];
+      if (lane == 0 && kS < sh) a.sk_out[r] = a.hashes[lbo + kS];
+      if (a.want_hashes)
+        for (int64_t b = lane; b < sh; b += 32) a.hashes[bo + b] = a.hashes[lbo + b];
+      for (int64_t f = sh; f < nb && (!dead || a.want_hashes || f <= kS);) {
+        const int len = (int)min((int64_t)(f == sh ? 1 : 32), nb - f);
+        const uint64_t d = lane < len ? __ldg(a.D + bo + f + lane) : 0;
+        uint64_t mine = 0;
+        for (int i = 0; i < len; ++i) {
+          h = chain_step(h, __shfl_sync(kFull, d, i));
+          if (lane == i) mine = h;
+        }
+        if (lane < len) {
+          if (a.want_hashes) a.hashes[bo + f + lane] = mine;
+          if (f + lane == kS) a.sk_out[r] = mine;
+        }
+        if (!dead) {
+          uint64_t x[W];
+          if (lane < len) {
+            probe_one<W>(a.tags, a.table, a.n_buckets, mine, x);
+          } else {
+#pragma unroll
+            for (int w = 0; w < W; ++w) x[w] = ~0ull;
+          }
+          __syncwarp();
+          dead = span(f, len, x);
+        }
         f += len;
-        continue;
-      }
-      const int64_t nfull = (F1 - f) >> 5;
-#pragma unroll
-      for (int w = 0; w < W; ++w) x[w] = first ? pre[w] : lane < nfull ? and_at(((f - bo) >> 5) + lane, w) : 0;
-      first = false;
-      bool stop = lane >= nfull;
-#pragma unroll
-      for (int w = 0; w < W; ++w) {
-        stop |= (x[w] & A[w]) != A[w];
-        if (w == gword && galive) stop |= !(x[w] & gbit);
-      }
-      const unsigned sm = __ballot_sync(kFull, stop);
-      const int j = sm ? __ffs(sm) - 1 : 32;
-      f += 32 * (int64_t)j;  // chunks that keep every alive run
-      if (galive) g = f - bo;
-      if (j < nfull && j < 32) {
-#pragma unroll
-        for (int w = 0; w < W; ++w) x[w] = mask_at(f - bo + lane, w);
-        dead = span(f - bo, 32, x);
-        f += 32;
       }
     }
     if (galive) g = nb;  // the global run reaches the last block
-    __syncwarp();
     // per instance (lanes = instances): c_i, then the decision
     int64_t best_cost = INT64_MAX;
     int32_t best = N;
@@ -1381,22 +1438,13 @@ __global__ void __launch_bounds__(kMatchWarps * 32, 5)
     }
     const int32_t s0 = DECIDE == kSession || DECIDE == kColoc ? (int32_t)(((int64_t)pol.rr_base + r) % N) : 0;
     const int64_t budget2 = DECIDE == kSession || DECIDE == kColoc ? 2 * (pol.d0 + pol.d1 * L) : 0;
-    int32_t* const out_c = summ + r * (N + 1);
+    int32_t* const out_c = a.summ + r * (N + 1);
 #pragma unroll
     for (int t = 0; t < CT; ++t) {
       const int i = 32 * t + lane;
       if (i >= N) break;
-      const int wi = i >> 6;
-      const uint64_t bi = 1ull << (i & 63);
-      uint64_t aw = 0;
-#pragma unroll
-      for (int w = 0; w < W; ++w) if (w == wi) aw = A[w];
-      int64_t ci = nb;
-      if (!(aw & bi)) {
-        for (int e = 0; e < ne; ++e)
-          if (ev_mask[e * W + wi] & bi) { ci = ev_pos[e]; break; }
-      }
-      out_c[i] = (int32_t)ci;  // every request's run ends (for the sequential variant)
+      const int64_t ci = c[t];
+      if (pol.summ) out_c[i] = c[t];
       if (DECIDE == kArgmin) {
         const int64_t gi = ci > g ? ci : g;
         const int64_t cost = w_load * load_s[i] + w_miss * (L - B * gi) + w_glob * B * (gi - ci);
@@ -1433,7 +1481,7 @@ __global__ void __launch_bounds__(kMatchWarps * 32, 5)
         }
       }
     }
-    if (lane == 0) out_c[N] = (int32_t)g;
+    if (pol.summ && lane == 0) out_c[N] = (int32_t)g;
     if (DECIDE == kBailian || DECIDE == kLMetric) {
 #pragma unroll
       for (int dd = 16; dd > 0; dd >>= 1) {
@@ -1516,9 +1564,9 @@ __global__ void __launch_bounds__(kMatchWarps * 32, 5)
   }
   // the group stage has read the group table: empty it for the next route
   // (it is zero from index creation before the first)
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < group_vecs;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.group_vecs;
        i += (int64_t)gridDim.x * blockDim.x)
-    groups[i] = make_uint4(0, 0, 0, 0);
+    a.groups[i] = make_uint4(0, 0, 0, 0);
 }
 
 // ---------------------------------------------------------------------------
@@ -2094,14 +2142,34 @@ int dispatch_digest(smetric_index* idx, const int32_t* d_tokens, int64_t n_token
   }
 }
 
-int launch_chain(smetric_index* idx, const int64_t* d_offsets, int32_t n, uint64_t* hashes,
-                 uint64_t* sk, bool pdl, cudaStream_t s) {
-  const unsigned grid = (unsigned)((n + kChainThreads - 1) / kChainThreads);
-  const uint64_t h_init = mix64(idx->cfg.hash_seed + kGamma);
-  idx->launches++;
-  return launch_k(k_chain, dim3(grid), dim3(kChainThreads), 0, s, pdl, d_offsets, idx->block_off, n,
-                  idx->cfg.block_size, idx->cfg.session_blocks, h_init, idx->batch_ok, idx->digest,
-                  hashes ? hashes : idx->hashes, sk);
+// Chain, shared prefixes and probe (W > 0), or the chain alone (W = 0): one CTA
+// per SM, a chain lane for each request a CTA owns (1 to 4 warps; more requests
+// share lanes). The ring's slots per lane fit 139 KB: 8 with one or two chain
+// warps, 4 with three or four.
+template <int W>
+int launch_chain_probe(ChainArgs a, int num_sms, cudaStream_t s, bool pdl) {
+  const int grid = (int)std::min<int64_t>(num_sms, a.n);
+  const int64_t per_cta = ((int64_t)a.n + grid - 1) / grid;
+  a.chain_warps = (int)std::max<int64_t>(1, std::min<int64_t>(kCpMaxChainWarps, (per_cta + 31) / 32));
+  a.slots = a.chain_warps <= 2 ? kCpMaxSlots : kCpMaxSlots / 2;
+  const size_t smem = (size_t)32 * a.chain_warps * a.slots * kCpRow;
+  if (cudaFuncSetAttribute(k_chain_probe<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return cuda_status(cudaErrorInvalidValue);
+  return launch_k(k_chain_probe<W>, dim3((unsigned)grid), dim3(cp_warps(W) * 32), smem, s, pdl, a);
+}
+
+// The arguments that every chain launch of an index has.
+ChainArgs chain_args(const smetric_index* idx, int32_t n, uint64_t* sk) {
+  ChainArgs a = {};
+  a.block_off = idx->block_off;
+  a.n = n;
+  a.S = idx->cfg.session_blocks;
+  a.h_init = mix64(idx->cfg.hash_seed + kGamma);
+  a.batch_ok = idx->batch_ok;
+  a.D = idx->digest;
+  a.sk_out = sk;
+  a.status = idx->status;
+  return a;
 }
 
 template <int W>
@@ -2112,38 +2180,37 @@ int launch_match(smetric_index* idx, const int64_t* d_offsets, int32_t n, const 
   const cudaEvent_t after_chain = ov ? ov->after_chain : nullptr;
   const int N = idx->cfg.num_instances;
   int rc;
+  // Short tails are left to the walk where the chain warps would have several
+  // lanes in use otherwise (with few requests an SM a tail chained after its
+  // leader only adds to the batch's time), and while the chain kernel can deal
+  // the rest out by k_lead's flags: 32 requests a thread, kCpRound a CTA.
+  const bool defer = n > 4 * idx->num_sms && n <= 32 * kCpWarps * 32 &&
+                     (n + idx->num_sms - 1) / idx->num_sms <= kCpRound;
+  // one byte a request, in the scratch words k_link_sessions uses for its keys
+  uint8_t* const flags = reinterpret_cast<uint8_t*>(idx->sk_tmp);
   {
-    // chain, group leaders and shared prefixes, and probe: one CTA per SM,
-    // a chain lane for each request a CTA owns (1 to 4 warps; more requests
-    // are taken in groups)
-    const int grid = idx->num_sms;
-    const int64_t per_cta = ((int64_t)n + grid - 1) / grid;
-    const int chain_warps = (int)std::max<int64_t>(1, std::min<int64_t>(kCpMaxChainWarps, (per_cta + 31) / 32));
-    const size_t smem = (size_t)chain_warps * 32 * kCpRingBytes;
-    // leader flags, one byte a request, in the scratch words k_link_sessions uses for its keys
-    uint8_t* const flags = reinterpret_cast<uint8_t*>(idx->sk_tmp);
     idx->launches++;
-    if ((rc = launch_k(k_lead, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, s, !idx->profiling,
+    if ((rc = launch_k(k_lead, dim3((unsigned)((n + 7) / 8)), dim3(256), 0, s, !idx->profiling,
                        (const int64_t*)idx->block_off, n, (const int32_t*)idx->batch_ok, (const uint64_t*)idx->digest,
-                       mix64(idx->cfg.hash_seed + kGamma), (const uint64_t*)idx->groups, group_slots_for(n) - 1,
-                       flags)))
+                       mix64(idx->cfg.hash_seed + kGamma), (const uint64_t*)idx->groups, group_slots_for(n) - 1, defer,
+                       idx->lead, idx->share, flags)))
       return rc;
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(k_chain_probe<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return cuda_status(cudaErrorInvalidValue);
+    ChainArgs a = chain_args(idx, n, sk);
+    a.chunk_off = idx->chunk_off;
+    a.hashes = hashes ? hashes : defer ? idx->hashes : nullptr;
+    a.share = idx->share;
+    a.active = flags;
+    a.deal = defer;
+    a.tags = idx->tags;
+    a.table = idx->table;
+    a.n_buckets = idx->n_buckets;
+    a.masks = idx->masks;
+    a.chunk_and = idx->chunk_and;
     idx->launches++;
-    if ((rc = launch_k(k_chain_probe<W>, dim3((unsigned)grid), dim3(kCpWarps * 32), smem, s, !idx->profiling,
-                       (const int64_t*)idx->block_off, (const int64_t*)idx->chunk_off, n, idx->cfg.session_blocks,
-                       mix64(idx->cfg.hash_seed + kGamma), (const int32_t*)idx->batch_ok,
-                       (const uint64_t*)idx->digest, hashes ? hashes : idx->hashes, sk, (const uint64_t*)idx->groups,
-                       group_slots_for(n) - 1, idx->lead, idx->share, (const uint8_t*)idx->tags,
-                       (const uint64_t*)idx->table, idx->n_buckets, idx->masks, idx->chunk_and,
-                       (const uint8_t*)flags, chain_warps, idx->status)))
-      return rc;
+    if ((rc = launch_chain_probe<W>(a, idx->num_sms, s, !idx->profiling))) return rc;
     if (after_chain && cudaEventRecord(after_chain, s) != cudaSuccess) return cuda_status(cudaErrorUnknown);
   }
   profile_mark(idx, kChainProbe, s);
-  const size_t smem = (size_t)N * sizeof(int64_t) + (size_t)kMatchWarps * N * (W + 1) * sizeof(uint64_t);
   const int64_t want = ((int64_t)n + kMatchWarps - 1) / kMatchWarps;
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)idx->num_sms * 8));
   // every request in one pass (members read their leaders' probes)
@@ -2151,16 +2218,41 @@ int launch_match(smetric_index* idx, const int64_t* d_offsets, int32_t n, const 
   const WalkKernel kerns[5] = {k_walk<W, kArgmin>, k_walk<W, kSession>, k_walk<W, kColoc>, k_walk<W, kBailian>,
                                k_walk<W, kLMetric>};
   const WalkKernel kern = kerns[pol.on];
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return cuda_status(cudaErrorInvalidValue);
   idx->launches++;
-  if ((rc = launch_k(kern, dim3((unsigned)grid), dim3(kMatchWarps * 32), smem, s, !idx->profiling, N,
-                     idx->cfg.block_size, d_offsets, idx->block_off, n, d_load, w.w_load, w.w_miss, w.w_glob,
-                     idx->masks, idx->chunk_and, (const int64_t*)idx->chunk_off, idx->batch_ok, idx->lead,
-                     idx->share, idx->summ, inst, lhit, ghit, reinterpret_cast<uint4*>(idx->groups),
-                     (int64_t)group_slots_for(n), pol)))
-    return rc;
+  WalkArgs a = {};
+  a.N = N;
+  a.B = idx->cfg.block_size;
+  a.S = idx->cfg.session_blocks;
+  a.off = d_offsets;
+  a.block_off = idx->block_off;
+  a.chunk_off = idx->chunk_off;
+  a.n = n;
+  a.load = d_load;
+  a.w_load = w.w_load;
+  a.w_miss = w.w_miss;
+  a.w_glob = w.w_glob;
+  a.masks = idx->masks;
+  a.chunk_and = idx->chunk_and;
+  a.batch_ok = idx->batch_ok;
+  a.lead = idx->lead;
+  a.share = idx->share;
+  a.summ = idx->summ;
+  a.inst_out = inst;
+  a.lhit_out = lhit;
+  a.ghit_out = ghit;
+  a.groups = reinterpret_cast<uint4*>(idx->groups);
+  a.group_vecs = (int64_t)group_slots_for(n);
+  if (defer) {
+    a.active = flags;
+    a.D = idx->digest;
+    a.hashes = hashes ? hashes : idx->hashes;
+    a.want_hashes = hashes != nullptr;
+    a.sk_out = sk;
+    a.tags = idx->tags;
+    a.table = idx->table;
+    a.n_buckets = idx->n_buckets;
+  }
+  if ((rc = launch_k(kern, dim3((unsigned)grid), dim3(kMatchWarps * 32), 0, s, !idx->profiling, a, pol))) return rc;
   return SMETRIC_OK;
 }
 
@@ -2242,7 +2334,10 @@ int route_common(smetric_index* idx, const int32_t* d_tokens, int64_t n_tokens, 
                              n_tokens / c.block_size, pol ? *pol : off_pol, s, ov)))
       return rc;
   } else {
-    if ((rc = launch_chain(idx, d_offsets, n, hashes, sk, !idx->profiling, s))) return rc;
+    ChainArgs a = chain_args(idx, n, sk);
+    a.hashes = hashes;
+    idx->launches++;
+    if ((rc = launch_chain_probe<0>(a, idx->num_sms, s, !idx->profiling))) return rc;
     profile_mark(idx, kChainProbe, s);
   }
   profile_mark(idx, kWalk, s);
@@ -2263,7 +2358,7 @@ int route_policy(smetric_index* idx, int mode, const int32_t* d_tokens, int64_t 
       p.reserved != 0)
     return SMETRIC_ERR_INVALID_ARG;
   if (n_requests > 0 && (!d_turn || !d_est_hit || !d_stick)) return SMETRIC_ERR_INVALID_ARG;
-  WalkPolicy pol;
+  WalkPolicy pol = {};
   pol.on = mode;
   pol.c_lin = p.c_lin;
   pol.c_att = p.c_att;
@@ -2388,7 +2483,7 @@ int pipeline_attach(smetric_index* x) {
   if (!p) return SMETRIC_ERR_OOM;
   RouteScratchSet& a = p->alt;
   bool ok = cudaMalloc(&a.block_off, (R + 1) * sizeof(int64_t)) == cudaSuccess &&
-            cudaMalloc(&a.digest, (nb + 2) * sizeof(uint64_t)) == cudaSuccess &&
+            cudaMalloc(&a.digest, nb * sizeof(uint64_t)) == cudaSuccess &&
             cudaMalloc(&a.hashes, nb * sizeof(uint64_t)) == cudaSuccess &&
             cudaMalloc(&a.masks, nb * W * sizeof(uint64_t)) == cudaSuccess &&
             cudaMalloc(&a.chunk_and, (max_blocks / 32 + R + 1) * W * sizeof(uint64_t)) == cudaSuccess &&
@@ -2545,8 +2640,10 @@ int smetric_route_batch_sequential(smetric_index* idx, const int32_t* d_tokens, 
                                    int64_t hashes_cap, int64_t* d_load_after, smetric_stream_t stream) {
   CallRange range("smetric_route_batch_sequential");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  WalkPolicy pol = {};
+  pol.summ = 1;
   int rc = route_common<true>(idx, d_tokens, n_tokens, d_offsets, n_requests, d_load, w, d_instance, d_local_hit,
-                              d_global_hit, d_session_key, d_block_hashes, hashes_cap, s);
+                              d_global_hit, d_session_key, d_block_hashes, hashes_cap, s, &pol);
   if (rc || n_requests == 0) return rc;
   k_seq<<<1, 32, 0, s>>>(idx->cfg.num_instances, idx->cfg.block_size, d_offsets, n_requests, d_load, w.w_load,
                          w.w_miss, w.w_glob, idx->summ, idx->batch_ok, d_instance, d_local_hit, d_global_hit,
@@ -2891,8 +2988,15 @@ extern "C" int smetric_block_hashes_noalloc(const int32_t* d_tokens, int64_t n_t
     }
     if (rc) return rc;
   }
-  const unsigned grid = (unsigned)((n_requests + kChainThreads - 1) / kChainThreads);
-  k_chain<<<grid, kChainThreads, 0, s>>>(d_offsets, block_off, n_requests, B, session_blocks,
-                                         mix64(hash_seed + kGamma), ok, digest, d_block_hashes, d_session_key);
-  return cuda_status(cudaGetLastError());
+  ChainArgs a = {};
+  a.block_off = block_off;
+  a.n = n_requests;
+  a.S = session_blocks;
+  a.h_init = mix64(hash_seed + kGamma);
+  a.batch_ok = ok;
+  a.D = digest;
+  a.hashes = d_block_hashes;
+  a.sk_out = d_session_key;
+  a.status = d_status;
+  return launch_chain_probe<0>(a, num_sms, s, false);
 }

@@ -23,7 +23,7 @@ __host__ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
 
 // The table is an array of buckets of kSlots = 15 slots. A bucket's 16-byte
 // tag group (in a tag array of its own) holds a one-byte tag per slot (0:
-// empty; otherwise 0x80 | low 7 key bits) and, in byte 15, the bucket's
+// empty; otherwise the low key byte, 1 for 0) and, in byte 15, the bucket's
 // overflow count: how many keys stored past this bucket probed through it
 // (saturating at 255, which then stays). Entries (key + tier-mask words) are
 // in the entry array, slot sl of bucket b at b * kSlots + sl. A key's home
@@ -38,57 +38,40 @@ __host__ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
 // read.
 constexpr int kBucket = 16;  // bytes of a bucket's tag group
 constexpr int kSlots = 15;   // slots of a bucket
-constexpr uint32_t kSlotBits = (1u << kSlots) - 1;
-
-// mix64 on 32-bit halves, for the serial chain where only latency counts:
-// the high word of each product is one three-input sum of the low-by-low
-// high half and the two cross products. Same value as mix64.
-__device__ __forceinline__ uint64_t mix64_halves(uint64_t z) {
-  uint32_t lo = (uint32_t)z, hi = (uint32_t)(z >> 32);
-  auto xs = [&](int s) {
-    lo ^= __funnelshift_r(lo, hi, s);
-    hi ^= hi >> s;
-  };
-  auto mul = [&](uint64_t c) {
-    const uint32_t cl = (uint32_t)c, ch = (uint32_t)(c >> 32);
-    const uint32_t x1 = lo * ch, x2 = hi * cl;
-    hi = __umulhi(lo, cl) + x1 + x2;
-    lo = lo * cl;
-  };
-  xs(30);
-  mul(0xBF58476D1CE4E5B9ull);
-  xs(27);
-  mul(0x94D049BB133111EBull);
-  xs(31);
-  return ((uint64_t)hi << 32) | lo;
-}
 
 __device__ __forceinline__ uint64_t home_bucket(uint64_t key, uint64_t n_buckets) {
   return __umul64hi(key, n_buckets);
 }
 
 __host__ __device__ __forceinline__ uint32_t key_tag(uint64_t key) {
-  return 0x80u | (uint32_t)(key & 0x7Fu);
+  const uint32_t t = (uint32_t)key & 0xFFu;
+  return t ? t : 1u;
 }
 
-// Bit s of the result is set where byte s of the 16 tag bytes equals `tag`.
-__device__ __forceinline__ uint32_t tag_match(uint4 t, uint32_t tag) {
+// The slots of a bucket whose tag equals `tag` (0: the empty ones), as a set
+// that next_slot takes apart; byte 15, the overflow count, is left out. Bit
+// 8 b + w stands for byte b of tag word w, slot 4 w + b: the zero bytes of
+// x ^ tag have their top bit set by an exact test per word, and the four words'
+// top bits go side by side, ~24 instructions for the 16 bytes (a per-byte
+// compare and gather took ~70; a probe runs this once or twice).
+__device__ __forceinline__ uint32_t slot_match(uint4 t, uint32_t tag) {
   const uint32_t rep = tag * 0x01010101u;
+  const uint32_t w[4] = {t.x ^ rep, t.y ^ rep, t.z ^ rep, t.w ^ rep};
   uint32_t m = 0;
-  const uint32_t w[4] = {t.x, t.y, t.z, t.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const uint32_t eq = __vcmpeq4(w[i], rep);  // 0xff in each equal byte
-    // gather the top bit of each byte into 4 bits
-    const uint32_t b = ((eq >> 7) & 1u) | ((eq >> 14) & 2u) | ((eq >> 21) & 4u) | ((eq >> 28) & 8u);
-    m |= b << (4 * i);
+    const uint32_t zero = ~(((w[i] & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | w[i]) & 0x80808080u;
+    m |= zero >> (7 - i);
   }
-  return m;
+  return m & ~(1u << 27);
 }
 
-// Bit s of the result is set where slot s's tag equals `tag` (byte 15, the
-// overflow count, left out).
-__device__ __forceinline__ uint32_t slot_match(uint4 t, uint32_t tag) { return tag_match(t, tag) & kSlotBits; }
+// Takes one slot out of a set that slot_match gave.
+__device__ __forceinline__ int next_slot(uint32_t& set) {
+  const int p = __ffs(set) - 1;
+  set &= set - 1;
+  return 4 * (p & 7) + (p >> 3);
+}
 
 // A bucket's overflow count (byte 15 of its tag group).
 __device__ __forceinline__ uint32_t overflow_count(uint4 t) { return t.w >> 24; }
@@ -110,9 +93,8 @@ __device__ __forceinline__ void latch_error(int32_t* status, int32_t code) {
 __host__ __device__ constexpr int entry_words(int W) { return W == 1 ? 2 : (W <= 3 ? 4 : 8); }
 
 // Route kernels, in launch order; names returned by smetric_profile_kernel_name.
-// kChainProbe is k_lead and k_chain_probe in a route (leader flags, then
-// chain, group stage and probe in one kernel) and k_chain in the calls that
-// only hash.
+// kChainProbe is k_lead and k_chain_probe in a route (group stage, then chain
+// and probe in one kernel) and the chain alone in the calls that only hash.
 enum RouteKernel { kPrep = 0, kDigest = 1, kChainProbe = 2, kWalk = 3, kNumRouteKernels = 4 };
 
 struct ProfileSlot {
@@ -165,8 +147,8 @@ struct smetric_index {
   uint64_t group_slots;  // power of two >= 2 * max_batch_requests
   int32_t* lead;       // max_batch_requests: the request whose masks a request shares
   int32_t* share;      // max_batch_requests: leading blocks taken from the leader
-  int32_t* summ;       // max_batch_requests * (num_instances + 1): a leader's run ends c_i, then g
-  uint64_t* sk_tmp;     // max_batch_requests: session keys nobody reads (session links); a route's leader flags
+  int32_t* summ;       // max_batch_requests * (num_instances + 1): run ends c_i, then g (the sequential variant)
+  uint64_t* sk_tmp;     // max_batch_requests: session keys nobody reads (session links); a route's k_lead marks
   int64_t* chunk_off;  // max_batch_requests + 1: first 32-block chunk of each request
   int32_t* batch_ok;   // device flag written by the prep kernel
   // staging for smetric_route_batch_host

@@ -48,8 +48,7 @@ __device__ __forceinline__ int64_t find_slot(const uint8_t* __restrict__ tags, c
                               : *reinterpret_cast<const uint4*>(tags + b * kBucket);
     uint32_t cand = slot_match(tv, tg);
     while (cand) {
-      const int sl = __ffs(cand) - 1;
-      cand &= cand - 1;
+      const int sl = next_slot(cand);
       const uint64_t slot = b * kSlots + sl;
       const uint64_t k = VOLATILE ? *reinterpret_cast<const volatile uint64_t*>(table + slot * ew)
                                   : table[slot * ew];
@@ -83,8 +82,7 @@ __device__ __forceinline__ bool insert_key(uint8_t* tags, uint64_t* table, int e
     const uint4 tv = load_tags_volatile(tags + b * kBucket);
     uint32_t cand = slot_match(tv, tg);
     while (cand) {
-      const int sl = __ffs(cand) - 1;
-      cand &= cand - 1;
+      const int sl = next_slot(cand);
       unsigned long long* e = reinterpret_cast<unsigned long long*>(table + (b * kSlots + sl) * ew);
       if (*reinterpret_cast<volatile unsigned long long*>(e) == key) {
         atomicOr(e + 1 + word, m);
@@ -93,8 +91,7 @@ __device__ __forceinline__ bool insert_key(uint8_t* tags, uint64_t* table, int e
     }
     uint32_t empty = slot_match(tv, 0);
     while (empty) {
-      const int sl = __ffs(empty) - 1;
-      empty &= empty - 1;
+      const int sl = next_slot(empty);
       unsigned long long* e = reinterpret_cast<unsigned long long*>(table + (b * kSlots + sl) * ew);
       const unsigned long long old = atomicCAS(e, (unsigned long long)kEmpty, (unsigned long long)key);
       if (old == kEmpty) {
