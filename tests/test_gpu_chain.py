@@ -7,7 +7,7 @@ import pytest
 torch = pytest.importorskip("torch")
 
 import oracle
-from gpu_util import assert_outputs_equal, gpu_hashes, gpu_route, make_index, populate_both
+from gpu_util import T, assert_outputs_equal, gpu_hashes, gpu_route, make_index, populate_both
 from pins import GAMMA, M64, _py_mix64, py_mix64_inverse
 from synth.traces import pack
 
@@ -106,3 +106,32 @@ def test_sentinel_in_the_middle_of_a_chain(at):
         assert int(o["block_hashes"][at]) == 2 + target
         assert_outputs_equal(g, o, ctx=f"sentinel at {at}")
         ix.close()
+
+
+@pytest.mark.parametrize("N", [1, 32, 33, 65, 128, 129, 256])
+@pytest.mark.parametrize("n", [1, 11, 12, 13, 37, 301])
+def test_sequential_stages_and_cost_widths(N, n):
+    """Batches around the stages of the sequential decision, instance counts
+    around its instances per lane, equal costs (the lowest instance), and
+    costs on both sides of 2^55, where the reductions change."""
+    rng = np.random.default_rng(1000 * N + n)
+    B = 4
+    pool = _tokens(rng, 400)
+    reqs = [np.concatenate([pool[:int(rng.integers(0, 300))], _tokens(rng, rng.integers(0, 40))]) for _ in range(n)]
+    ix = make_index(N, B, 2)
+    ox = oracle.OracleIndex(N)
+    populate_both(ix, ox, {t: [pool[:int(rng.integers(0, 400))]] for t in range(-1, min(N, 9))}, B)
+    tok, off = pack(reqs)
+    same = np.full(N, 7)
+    for w, load in (((1, 4, 2), same), ((0, 0, 0), same), ((1, 4, 2), rng.integers(0, 300, size=N)),
+                    ((2 ** 20, 2 ** 20, 1), (1 << 40) - rng.integers(0, 500, size=N)),
+                    ((2 ** 20, 3, 2 ** 20), np.full(N, 1 << 40)), ((2 ** 15, 4, 2), np.full(N, (1 << 40) - 1)),
+                    ((2 ** 15 - 1, 4, 2), np.full(N, (1 << 40) - 1))):
+        load = np.asarray(load, np.int64)
+        out = ix.route_batch_sequential(T(tok), T(off), T(load), w)
+        ix.check()
+        o = ox.route_batch_sequential(B, 2, 0, tok, off, load, *w)
+        g = {k: v.cpu().numpy() for k, v in out.items()}
+        assert_outputs_equal(g, o, fields=("instance", "local_hit", "global_hit", "session_key", "load_after"),
+                             ctx=f"N={N} n={n} w={w}")
+    ix.close()
