@@ -413,8 +413,9 @@ int smetric_route_commit_batch(smetric_index* idx, const int32_t* d_tokens, int6
  * smetric_index_clear): keys already in them are not tracked. Synchronises
  * the device; any earlier recency state is dropped. Device memory: 16 B per
  * capped block (two record buffers), plus 16 B x 2 x max_blocks of touch
- * lists, 16 B x 8 x max_blocks of per-batch sets and a byte per record and
- * touch (max_blocks = max_batch_tokens / B).
+ * and eviction lists, 16 B x 8 x max_blocks of per-batch sets, 12 B x
+ * max_blocks of their filters and the touches' places in them, and a bit per
+ * record and touch (max_blocks = max_batch_tokens / B).
  * Errors: a negative cap or one above 2^40 (INVALID_ARG), an allocation
  * failure (OOM: the LRU is off then). */
 int smetric_index_set_lru(smetric_index* idx, int64_t local_cap, int64_t global_cap);

@@ -44,6 +44,8 @@
 #include <cstring>
 
 #include "smetric_impl.cuh"
+#include "commit.cuh"
+#include "launch.cuh"
 
 using namespace smetric;
 
@@ -51,12 +53,6 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-// Programmatic dependent launch: a route kernel launched with programmatic
-// stream serialisation is set up while its predecessor still runs and waits
-// here until that predecessor has finished and its writes are visible (a
-// no-op for an ordinary launch). No kernel triggers its successor early:
-// successors waiting on the SMs during a kernel's run measured slower.
-__device__ __forceinline__ void pdl_enter() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 constexpr int kChunk = 32;        // blocks per digest task (one per lane)
 constexpr int kDigestWarps = 8;   // most warps per digest CTA
 constexpr int kTmaWarps = 24;     // warps per TMA digest CTA (two CTAs per SM)
@@ -2140,39 +2136,14 @@ __global__ void __launch_bounds__(1024)
 // commit
 // ---------------------------------------------------------------------------
 
-// Checks of a batch to commit and the queue drain: one CTA checks every
-// request's instance (in [-1, N)) and local hit (in [0, L_r]); a bad value
-// clears the batch flag, so that nothing is committed and the loads stay as
-// they were. Otherwise, with `load`, it sums per instance the tokens each
-// request routed there must prefill or fetch (L_r - local hit) and sets
-// load_i <- (load_i + that sum) >> 1. Integer sums, so the order of the
-// atomics does not matter.
+// Checks of a batch to commit and the queue drain, on an index without an LRU
+// (with one, its first kernel does both).
 __global__ void __launch_bounds__(1024)
     k_drain(const int64_t* __restrict__ off, int32_t n, int N, const int32_t* __restrict__ instance,
             const int32_t* __restrict__ local_hit, int32_t* __restrict__ batch_ok,
             int64_t* __restrict__ load, int32_t* status) {
-  __shared__ unsigned long long acc[SMETRIC_MAX_INSTANCES];
-  __shared__ int bad;
-  if (threadIdx.x == 0) bad = 0;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) acc[i] = 0;
-  __syncthreads();
-  if (!*batch_ok) return;  // invalid offsets
-  for (int64_t r = threadIdx.x; r < n; r += blockDim.x) {
-    const int32_t i = instance[r];
-    const int64_t L = off[r + 1] - off[r], h = local_hit ? local_hit[r] : 0;
-    if (i < -1 || i >= N || h < 0 || h > L) { bad = 1; continue; }
-    if (i >= 0 && load) atomicAdd(&acc[i], (unsigned long long)(L - h));
-  }
-  __syncthreads();
-  if (bad) {
-    if (threadIdx.x == 0) {
-      *batch_ok = 0;
-      latch_error(status, SMETRIC_ERR_INVALID_ARG);
-    }
-    return;
-  }
-  if (load)
-    for (int i = threadIdx.x; i < N; i += blockDim.x) load[i] = (load[i] + (int64_t)acc[i]) >> 1;
+  pdl_enter();
+  drain_batch(off, n, N, instance, local_hit, batch_ok, load, status);
 }
 
 // ---------------------------------------------------------------------------
@@ -2187,24 +2158,6 @@ void profile_mark(smetric_index* idx, int k, cudaStream_t s);
 struct Overlap {
   cudaEvent_t after_chain;
 };
-
-// Launches a route kernel; with pdl the launch may begin while the previous
-// kernel on the stream is still running (the kernel waits in pdl_enter).
-template <typename... KArgs, typename... Args>
-int launch_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl,
-             Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = pdl ? attr : nullptr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  return cuda_status(cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...));
-}
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
@@ -2786,15 +2739,15 @@ int commit_common(smetric_index* idx, const int64_t* d_offsets, int32_t n_reques
     idx->launches++;
     if ((rc = cuda_status(cudaGetLastError()))) return rc;
   }
+  const bool global = (flags & SMETRIC_COMMIT_GLOBAL) != 0;
+  if (idx->lru)
+    return lru_commit(idx, d_offsets, d_instance, d_local_hit, d_block_hashes, n_requests, global, d_load, s);
   // the checks (and the drain) first: a bad output commits nothing
-  k_drain<<<1, 1024, 0, s>>>(d_offsets, n_requests, c.num_instances, d_instance, d_local_hit, idx->batch_ok,
-                             d_load, idx->status);
   idx->launches++;
-  if ((rc = cuda_status(cudaGetLastError()))) return rc;
-  if ((rc = launch_commit(idx, d_instance, d_block_hashes, n_requests, c.max_batch_tokens / c.block_size,
-                          (flags & SMETRIC_COMMIT_GLOBAL) != 0, s)))
+  if ((rc = launch_k(k_drain, dim3(1), dim3(1024), 0, s, true, d_offsets, n_requests, c.num_instances, d_instance,
+                     d_local_hit, idx->batch_ok, d_load, idx->status)))
     return rc;
-  return lru_commit(idx, d_instance, d_block_hashes, n_requests, (flags & SMETRIC_COMMIT_GLOBAL) != 0, s);
+  return launch_commit(idx, d_instance, d_block_hashes, n_requests, c.max_batch_tokens / c.block_size, global, s);
 }
 
 }  // namespace

@@ -119,7 +119,11 @@ struct LruState {
   uint64_t* touches = nullptr;            // 2 * max_blocks: the batch's touches, tier after tier
   uint64_t* set = nullptr;                // set_entries (key, last touch + 1) pairs
   int64_t set_entries = 0;
-  uint8_t* keep = nullptr;                // max_tiles * kLruTile flags
+  uint32_t* where = nullptr;              // 2 * max_blocks: each touch's entry in its tier's set
+  uint32_t* filter = nullptr;             // filter_words: a bit per hash of a touched key, tier after tier
+  int64_t filter_words = 0;
+  uint32_t* keep = nullptr;               // max_tiles * kLruTile flags, one bit each
+  uint64_t* evicted = nullptr;            // 2 * max_blocks: the batch's evicted keys, tier after tier
   int64_t* tile_cnt = nullptr;            // max_tiles + 1, then their exclusive scan
   int64_t* tile_off = nullptr;
   int64_t max_tiles = 0;
@@ -175,10 +179,11 @@ int cuda_status(cudaError_t e);
 // (and the global tier); block_off must hold the batch's block offsets.
 int launch_commit(smetric_index* idx, const int32_t* d_instance, const uint64_t* d_hashes, int32_t n,
                   int64_t max_blocks, bool global, cudaStream_t s);
-// After a commit's inserts: the capped tiers' recency lists take the batch's
-// touches and evict what exceeds each cap (no-op without an LRU).
-int lru_commit(smetric_index* idx, const int32_t* d_instance, const uint64_t* d_hashes, int32_t n, bool global,
-               cudaStream_t s);
+// The same on an index with an LRU, with the batch's checks and the queue drain
+// before it (drain_batch): then the capped tiers' recency lists take the
+// batch's touches and evict what exceeds each cap.
+int lru_commit(smetric_index* idx, const int64_t* d_offsets, const int32_t* d_instance, const int32_t* d_local_hit,
+               const uint64_t* d_hashes, int32_t n, bool global, int64_t* d_load, cudaStream_t s);
 // Empties every recency list (after the table is cleared).
 int lru_reset(smetric_index* idx, cudaStream_t s);
 // Frees the LRU state.

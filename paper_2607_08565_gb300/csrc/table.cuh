@@ -60,18 +60,42 @@ __device__ __forceinline__ int64_t find_slot(const uint8_t* __restrict__ tags, c
   return -1;
 }
 
-// Sets tier bit m of mask word `word` of `key`, taking a slot if the key is
-// new. Pass 1 looks the key up; pass 2 walks from the home bucket again and,
-// in each bucket, first takes the key if a concurrent inserter has just
-// placed it there, then tries each empty slot with a CAS on its key word.
-// The winner publishes the tag after a fence and counts itself in every
-// bucket it passed. A CAS that fails on this very key (claimed, tag not yet
-// published) uses that slot. Returns false when no slot was found.
+// Tier bits to set in one key's entry: m[0] in mask word word[0], and m[1] (0:
+// none) in word[1], another word.
+struct TierBits {
+  int word[2];
+  unsigned long long m[2];
+};
+
+__device__ __forceinline__ TierBits tier_bits(int bit) { return {{bit >> 6, 0}, {1ull << (bit & 63), 0ull}}; }
+__device__ __forceinline__ TierBits tier_bits(int a, int b) {
+  if ((a >> 6) == (b >> 6)) return {{a >> 6, 0}, {(1ull << (a & 63)) | (1ull << (b & 63)), 0ull}};
+  return {{a >> 6, b >> 6}, {1ull << (a & 63), 1ull << (b & 63)}};
+}
+
+// ORs the bits into entry e (looking first whether they are set took longer:
+// 57 us instead of 54 for 1.4M pairs of which two thirds were in the index).
+__device__ __forceinline__ void set_bits(unsigned long long* e, const TierBits& b) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    if (b.m[i] == 0ull) continue;
+    unsigned long long* const w = e + 1 + b.word[i];
+    atomicOr(w, b.m[i]);
+  }
+}
+
+// Sets tier bits of `key`, taking a slot if the key is new. Pass 1 looks the
+// key up; pass 2 walks from the home bucket again and, in each bucket, first
+// takes the key if a concurrent inserter has just placed it there, then tries
+// each empty slot with a CAS on its key word. The winner publishes the tag
+// after a fence and counts itself in every bucket it passed. A CAS that fails
+// on this very key (claimed, tag not yet published) uses that slot. Returns
+// false when no slot was found.
 __device__ __forceinline__ bool insert_key(uint8_t* tags, uint64_t* table, int ew, uint64_t n_buckets,
-                                           uint64_t key, int word, unsigned long long m) {
+                                           uint64_t key, const TierBits& bits) {
   const int64_t found = find_slot<true>(tags, table, ew, n_buckets, key);
   if (found >= 0) {
-    atomicOr(reinterpret_cast<unsigned long long*>(table + found * ew) + 1 + word, m);
+    set_bits(reinterpret_cast<unsigned long long*>(table + found * ew), bits);
     return true;
   }
   const uint32_t tg = key_tag(key);
@@ -85,7 +109,7 @@ __device__ __forceinline__ bool insert_key(uint8_t* tags, uint64_t* table, int e
       const int sl = next_slot(cand);
       unsigned long long* e = reinterpret_cast<unsigned long long*>(table + (b * kSlots + sl) * ew);
       if (*reinterpret_cast<volatile unsigned long long*>(e) == key) {
-        atomicOr(e + 1 + word, m);
+        set_bits(e, bits);
         return true;
       }
     }
@@ -101,11 +125,11 @@ __device__ __forceinline__ bool insert_key(uint8_t* tags, uint64_t* table, int e
           overflow_add(tags, p, +1);
           if (++p == n_buckets) p = 0;
         }
-        atomicOr(e + 1 + word, m);
+        set_bits(e, bits);
         return true;
       }
       if (old == key) {
-        atomicOr(e + 1 + word, m);
+        set_bits(e, bits);
         return true;
       }
     }
