@@ -2035,8 +2035,101 @@ __global__ void __launch_bounds__(256)
 // session links
 // ---------------------------------------------------------------------------
 
+// A request's parent is sought among the requests of its user's turn before:
+// k_link_turns lists the requests of each (user, turn) and k_link_parents goes
+// through the list that a request's parent must be in, comparing one hash per
+// entry. In a trace a list has one request or a few; a request whose list is
+// longer than kLinkList is marked instead (parent -2) and found by its prefixes
+// in three more kernels, which return at once when there is none. 8,192
+// requests of 750 blocks, lists of one: 10 us instead of 156 for a thread per
+// (request, prefix length).
+constexpr int kLinkList = 64;   // entries, a dependent read each
+constexpr int32_t kLinkMarked = -2;
+
+struct LinkState {
+  int32_t marked;  // some request is marked
+  int32_t deep;    // some chain of parents is longer than kLinkHops
+};
+
+__device__ __forceinline__ uint64_t turn_key(int64_t user, int64_t turn) {
+  const uint64_t x = mix64(mix64((uint64_t)user ^ kGamma) ^ (uint64_t)turn);
+  return x ? x : 1;
+}
+
+// Thread per request p: to the front of its (user, turn)'s list. A table entry
+// is the turn's fingerprint, the list's head (request + 1) and its length.
+__global__ void __launch_bounds__(256)
+    k_link_turns(int32_t n, const int32_t* __restrict__ batch_ok, const int64_t* __restrict__ users,
+                 const int32_t* __restrict__ turns, uint64_t* __restrict__ table, uint64_t gmask,
+                 int32_t* __restrict__ next, LinkState* state) {
+  pdl_enter();
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p == 0) *state = LinkState{0, 0};
+  if (p >= n || !*batch_ok) return;
+  const uint64_t key = turn_key(users[p], turns[p]);
+  uint64_t s = key & gmask;
+  for (uint64_t t = 0; t <= gmask; ++t) {
+    unsigned long long* const slot = reinterpret_cast<unsigned long long*>(table + 2 * s);
+    const unsigned long long old = atomicCAS(slot, 0ull, (unsigned long long)key);
+    if (old == 0ull || old == key) {
+      int32_t* const list = reinterpret_cast<int32_t*>(slot + 1);
+      next[p] = atomicExch(list, (int32_t)p + 1);
+      atomicAdd(list + 1, 1);
+      return;
+    }
+    s = (s + 1) & gmask;
+  }
+}
+
+// Thread per request r: the latest earlier request on the list of (user_r,
+// turn_r - 1) whose last block is r's block there. (A fingerprint may stand for
+// several turns: user and turn are compared.)
+__global__ void __launch_bounds__(256)
+    k_link_parents(const int64_t* __restrict__ block_off, int32_t n, const int32_t* __restrict__ batch_ok,
+                   const uint64_t* __restrict__ H, const int64_t* __restrict__ users,
+                   const int32_t* __restrict__ turns, const uint64_t* __restrict__ table, uint64_t gmask,
+                   const int32_t* __restrict__ next, int32_t* __restrict__ parent, int32_t* __restrict__ mark,
+                   LinkState* state) {
+  pdl_enter();
+  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= n || !*batch_ok) return;
+  const int64_t user = users[r], turn = (int64_t)turns[r] - 1;
+  const int64_t bo = __ldg(block_off + r), nb = __ldg(block_off + r + 1) - bo;
+  int32_t best = -1;
+  const uint64_t key = turn_key(user, turn);
+  uint64_t s = key & gmask;
+  for (uint64_t t = 0; t <= gmask; ++t) {
+    const ulonglong2 e = __ldg(reinterpret_cast<const ulonglong2*>(table + 2 * s));
+    if (e.x == 0) break;
+    if (e.x == key) {
+      if ((int32_t)(e.y >> 32) > kLinkList) {
+        best = kLinkMarked;
+        state->marked = 1;
+        break;
+      }
+      for (int32_t p = (int32_t)(uint32_t)e.y - 1; p >= 0; p = __ldg(next + p) - 1) {
+        if (p >= r || p <= best || users[p] != user || (int64_t)turns[p] != turn) continue;
+        const int64_t pbo = __ldg(block_off + p), k = __ldg(block_off + p + 1) - pbo;
+        if (k <= nb && (k == 0 || __ldg(H + pbo + k - 1) == __ldg(H + bo + k - 1))) best = p;
+      }
+      break;
+    }
+    s = (s + 1) & gmask;
+  }
+  parent[r] = best;
+  mark[r] = best;  // (the mark outlives a parent found later; the session output until it is written)
+}
+
+// With marked requests: empties the table for its use as a multi-map.
+__global__ void __launch_bounds__(256) k_link_clear(const LinkState* state, uint4* __restrict__ table, int64_t vecs) {
+  pdl_enter();
+  if (!state->marked) return;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < vecs; i += (int64_t)gridDim.x * blockDim.x)
+    table[i] = make_uint4(0, 0, 0, 0);
+}
+
 // Fingerprint of (user, turn, number of blocks, last block hash) for the
-// session-link table; 0 marks an empty slot.
+// multi-map; 0 marks an empty slot.
 __device__ __forceinline__ uint64_t link_key(int64_t user, int64_t turn, int64_t nb, uint64_t last) {
   uint64_t x = mix64((uint64_t)user ^ kGamma);
   x = mix64(x ^ (uint64_t)turn);
@@ -2045,16 +2138,16 @@ __device__ __forceinline__ uint64_t link_key(int64_t user, int64_t turn, int64_t
   return x ? x : 1;
 }
 
-// Thread per request p: (key, p) into the table (a multi-map: every request
-// takes its own slot), and parent[p] = -1.
+// With marked requests, thread per request p: (key, p) into the table (a
+// multi-map: every request takes its own slot).
 __global__ void __launch_bounds__(256)
     k_link_insert(const int64_t* __restrict__ block_off, int32_t n, const int32_t* __restrict__ batch_ok,
                   const uint64_t* __restrict__ H, const int64_t* __restrict__ users,
                   const int32_t* __restrict__ turns, uint64_t* __restrict__ table, uint64_t gmask,
-                  int32_t* __restrict__ parent) {
+                  const LinkState* state) {
+  pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n || !*batch_ok) return;
-  parent[p] = -1;
+  if (p >= n || !*batch_ok || !state->marked) return;
   const int64_t bo = block_off[p], nb = block_off[p + 1] - bo;
   const uint64_t key = link_key(users[p], turns[p], nb, nb ? H[bo + nb - 1] : 0);
   uint64_t s = key & gmask;
@@ -2068,16 +2161,18 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// Thread per (request r, prefix length k <= n_r): the latest earlier request
-// of r's user, of turn turn_r - 1, with exactly k blocks, the last equal to
-// r's block k - 1, raises parent[r] to it. Candidates from the table are
-// checked field by field.
+// Thread per (marked request r, prefix length k <= n_r): the latest earlier
+// request of r's user, of turn turn_r - 1, with exactly k blocks, the last equal
+// to r's block k - 1, raises parent[r] to it (any request is above the mark; one
+// without a parent keeps it). Candidates from the table are checked field by
+// field.
 __global__ void __launch_bounds__(256)
     k_link_find(const int64_t* __restrict__ block_off, int32_t n, const int32_t* __restrict__ batch_ok,
                 const uint64_t* __restrict__ H, const int64_t* __restrict__ users,
                 const int32_t* __restrict__ turns, const uint64_t* __restrict__ table, uint64_t gmask,
-                int32_t* __restrict__ parent) {
-  if (!*batch_ok) return;
+                int32_t* parent, const int32_t* __restrict__ mark, const LinkState* state) {
+  pdl_enter();
+  if (!*batch_ok || !state->marked) return;
   const int64_t total = block_off[n] + n;  // sum over r of n_r + 1
   int32_t r = 0;
   for (int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; f < total;
@@ -2088,6 +2183,7 @@ __global__ void __launch_bounds__(256)
       if (__ldg(block_off + mid) + mid <= f) lo = mid; else hi = mid;
     }
     r = lo;
+    if (mark[r] != kLinkMarked) continue;
     const int64_t bo = __ldg(block_off + r), k = f - (bo + r);
     const int64_t user = users[r], turn = (int64_t)turns[r] - 1;
     const uint64_t last = k ? __ldg(H + bo + k - 1) : 0;
@@ -2110,26 +2206,60 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// One CTA: session[r] = the head of r's chain of parents (pointer jumping;
-// parents are earlier requests, so every chain ends), then the link table
-// emptied for the next route.
+// Thread per request: up the chain of parents, kLinkHops of them at most; then
+// session[r] is the head, or an ancestor on the way to it. (Parents are earlier
+// requests, so every chain ends.) A parent left at the mark is none.
+constexpr int kLinkHops = 64;
+__global__ void __launch_bounds__(256)
+    k_link_chase(int32_t n, const int32_t* __restrict__ batch_ok, const int32_t* __restrict__ parent,
+                 int32_t* __restrict__ session, LinkState* state) {
+  pdl_enter();
+  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= n || !*batch_ok) return;
+  int32_t s = (int32_t)r;
+  for (int k = 0; k < kLinkHops; ++k) {
+    const int32_t p = __ldg(parent + s);
+    if (p < 0) break;
+    s = p;
+  }
+  if (__ldg(parent + s) >= 0) state->deep = 1;
+  session[r] = s;
+}
+
+// CTA 0: the heads of longer chains by pointer jumping (session[r] an ancestor
+// of r throughout), -1 everywhere after invalid offsets, and no parent where
+// one is still marked. The other CTAs empty the table for the next call.
 __global__ void __launch_bounds__(1024)
     k_link_heads(int32_t n, const int32_t* __restrict__ batch_ok, int32_t* __restrict__ parent,
-                 int32_t* __restrict__ session, uint4* __restrict__ table, int64_t table_vecs) {
-  if (*batch_ok) {
-    for (int32_t r = threadIdx.x; r < n; r += blockDim.x) session[r] = parent[r] < 0 ? r : parent[r];
-    __syncthreads();
-    for (int64_t span = 1; span < n; span <<= 1) {
-      for (int32_t r = threadIdx.x; r < n; r += blockDim.x) {
-        const int32_t a = session[r];
-        session[r] = session[a];  // an ancestor either way: the heads are reached all the same
-      }
-      __syncthreads();
-    }
-  } else {  // invalid offsets: no links
-    for (int32_t r = threadIdx.x; r < n; r += blockDim.x) { parent[r] = -1; session[r] = -1; }
+                 int32_t* __restrict__ session, uint4* __restrict__ table, int64_t table_vecs,
+                 const LinkState* state) {
+  pdl_enter();
+  if (blockIdx.x > 0) {
+    for (int64_t i = (int64_t)(blockIdx.x - 1) * blockDim.x + threadIdx.x; i < table_vecs;
+         i += (int64_t)(gridDim.x - 1) * blockDim.x)
+      table[i] = make_uint4(0, 0, 0, 0);
+    return;
   }
-  for (int64_t i = threadIdx.x; i < table_vecs; i += blockDim.x) table[i] = make_uint4(0, 0, 0, 0);
+  if (!*batch_ok) {
+    for (int32_t r = threadIdx.x; r < n; r += blockDim.x) { parent[r] = -1; session[r] = -1; }
+    return;
+  }
+  if (state->deep) {
+    for (int64_t span = 1; span < n; span <<= 1) {
+      int moved = 0;
+      for (int32_t r = threadIdx.x; r < n; r += blockDim.x) {
+        const int32_t a = session[r], b = session[a];
+        if (a != b) {
+          session[r] = b;  // an ancestor either way: the heads are reached all the same
+          moved = 1;
+        }
+      }
+      if (!__syncthreads_or(moved)) break;
+    }
+  }
+  if (state->marked)
+    for (int32_t r = threadIdx.x; r < n; r += blockDim.x)
+      if (parent[r] == kLinkMarked) parent[r] = -1;
 }
 
 // ---------------------------------------------------------------------------
@@ -2933,17 +3063,32 @@ int smetric_link_sessions(smetric_index* idx, const int32_t* d_tokens, int64_t n
                                 n_tokens / idx->cfg.block_size, s)))
     return rc;
   const uint64_t gmask = group_slots_for(n_requests) - 1;
-  const unsigned g = (unsigned)((n_requests + 255) / 256);
-  k_link_insert<<<g, 256, 0, s>>>(idx->block_off, n_requests, idx->batch_ok, idx->hashes, d_users, d_turns,
-                                  idx->groups, gmask, d_parent);
+  const dim3 g((unsigned)((n_requests + 255) / 256)), t(256);
   const int64_t want = (n_tokens / idx->cfg.block_size + n_requests + 255) / 256;
-  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)idx->num_sms * 8));
-  k_link_find<<<grid, 256, 0, s>>>(idx->block_off, n_requests, idx->batch_ok, idx->hashes, d_users, d_turns,
-                                   idx->groups, gmask, d_parent);
-  k_link_heads<<<1, 1024, 0, s>>>(n_requests, idx->batch_ok, d_parent, d_session,
-                                  reinterpret_cast<uint4*>(idx->groups), (int64_t)(gmask + 1));
-  idx->launches += 3;
-  return cuda_status(cudaGetLastError());
+  const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)idx->num_sms * 8)));
+  const int64_t* const bo = idx->block_off;
+  const int32_t* const ok = idx->batch_ok;
+  const uint64_t* const H = idx->hashes;
+  uint64_t* const table = idx->groups;
+  int32_t* const next = idx->lead;  // per request: the next of its turn's list
+  LinkState* const st = reinterpret_cast<LinkState*>(idx->share);
+  uint4* const vecs = reinterpret_cast<uint4*>(table);
+  idx->launches += 7;
+  if ((rc = launch_k(k_link_turns, g, t, 0, s, true, n_requests, ok, d_users, d_turns, table, gmask, next, st)) ||
+      (rc = launch_k(k_link_parents, g, t, 0, s, true, bo, n_requests, ok, H, d_users, d_turns,
+                     (const uint64_t*)table, gmask, (const int32_t*)next, d_parent, d_session, st)) ||
+      (rc = launch_k(k_link_clear, dim3((unsigned)idx->num_sms), t, 0, s, true, (const LinkState*)st, vecs,
+                     (int64_t)(gmask + 1))) ||
+      (rc = launch_k(k_link_insert, g, t, 0, s, true, bo, n_requests, ok, H, d_users, d_turns, table, gmask,
+                     (const LinkState*)st)) ||
+      (rc = launch_k(k_link_find, grid, t, 0, s, true, bo, n_requests, ok, H, d_users, d_turns,
+                     (const uint64_t*)table, gmask, d_parent, (const int32_t*)d_session, (const LinkState*)st)) ||
+      (rc = launch_k(k_link_chase, g, t, 0, s, true, n_requests, ok, (const int32_t*)d_parent, d_session, st)) ||
+      (rc = launch_k(k_link_heads, dim3((unsigned)std::min<int64_t>(1 + ((int64_t)gmask + 1024) / 1024, idx->num_sms)),
+                     dim3(1024), 0, s, true, n_requests, ok, d_parent, d_session, vecs, (int64_t)(gmask + 1),
+                     (const LinkState*)st)))
+    return rc;
+  return SMETRIC_OK;
 }
 
 int smetric_block_hashes(smetric_index* idx, const int32_t* d_tokens, int64_t n_tokens,
