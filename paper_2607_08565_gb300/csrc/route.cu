@@ -73,9 +73,28 @@ __device__ __forceinline__ int64_t warp_incl_scan(int64_t v, int lane) {
   return v;
 }
 
-constexpr int kPrepRounds = 8;  // rounds of 32 consecutive requests per warp per pass
+constexpr int kPrepThreads = 1024;
+constexpr int kPrepRounds = 8;  // rounds of 32 consecutive requests per warp
+constexpr int kPrepPass = kPrepThreads * kPrepRounds;  // requests a CTA scans at a time
+constexpr int64_t kPrepMaxCtas = 128;  // past 128 passes a CTA takes several
 
-__global__ void __launch_bounds__(1024) k_prep(const int64_t* __restrict__ off, int32_t n,
+// CTA j scans the j-th stretch of requests (a pass of kPrepPass while there are
+// no more than kPrepMaxCtas of them), after adding up the counts of all
+// requests before it by itself: reading 8 bytes a request again costs less than
+// waiting for another CTA, and what it costs is mostly the latency of a load.
+// The last CTA has seen every request then: it alone checks the batch, writes
+// the totals and the batch's flag. 32,768 requests: 16.5 us; 30 with one CTA
+// that took its passes one after another.
+inline int64_t prep_passes(int64_t n) {  // of one CTA
+  const int64_t passes = std::max<int64_t>(1, (n + kPrepPass - 1) / kPrepPass);
+  return (passes + kPrepMaxCtas - 1) / kPrepMaxCtas;
+}
+inline unsigned prep_grid(int64_t n) {
+  const int64_t stretch = prep_passes(n) * kPrepPass;
+  return (unsigned)std::max<int64_t>(1, (n + stretch - 1) / stretch);
+}
+
+__global__ void __launch_bounds__(kPrepThreads) k_prep(int passes, const int64_t* __restrict__ off, int32_t n,
                                               int64_t n_tokens, int B, const int64_t* __restrict__ load,
                                               int n_load, int64_t* __restrict__ block_off,
                                               int64_t* __restrict__ chunk_off, int32_t* batch_ok,
@@ -85,31 +104,48 @@ __global__ void __launch_bounds__(1024) k_prep(const int64_t* __restrict__ off, 
                                               const int64_t* __restrict__ aux1 = nullptr, int64_t aux1_max = 0) {
   constexpr int NS = 2;  // scans: full blocks, and 32-block chunks (when chunk_off is wanted)
   constexpr int R = kPrepRounds;
-  __shared__ int64_t warp_tot[NS][32];
+  __shared__ int64_t warp_tot[NS][32], warp_before[NS][32];
   __shared__ int64_t pass_tot[NS];
   __shared__ int bad_all;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const bool last = blockIdx.x == gridDim.x - 1;
   if (tid == 0) bad_all = 0;
   __syncthreads();
   int bad = 0;  // bit 0: invalid offsets, bit 1: out-of-range length or load
-  for (int i = tid; i < n_load; i += blockDim.x) {
-    const int64_t v = load[i];
-    if (v < 0 || v > max_load) bad |= 2;
-    if (aux0 && (aux0[i] < 0 || aux0[i] > aux0_max)) bad |= 2;  // further per-instance inputs
-    if (aux1 && (aux1[i] < 0 || aux1[i] > aux1_max)) bad |= 2;
-  }
-  if (est_hit)  // the policy's expected hits, each in [0, 2^31)
-    for (int64_t r = tid; r < n; r += blockDim.x) {
-      const int64_t v = est_hit[r];
-      if (v < 0 || v > (int64_t)INT32_MAX) bad |= 2;
+  if (last) {
+    for (int i = tid; i < n_load; i += blockDim.x) {
+      const int64_t v = load[i];
+      if (v < 0 || v > max_load) bad |= 2;
+      if (aux0 && (aux0[i] < 0 || aux0[i] > aux0_max)) bad |= 2;  // further per-instance inputs
+      if (aux1 && (aux1[i] < 0 || aux1[i] > aux1_max)) bad |= 2;
     }
-  // A pass gives each warp R rounds of 32 consecutive requests (lane = request),
+    if (est_hit)  // the policy's expected hits, each in [0, 2^31)
+      for (int64_t r = tid; r < n; r += blockDim.x) {
+        const int64_t v = est_hit[r];
+        if (v < 0 || v > (int64_t)INT32_MAX) bad |= 2;
+      }
+  }
+  // full blocks of a request from its two offsets, and their checks
+  auto blocks = [&](int64_t a, int64_t b) -> uint32_t {
+    if (a < 0 || b < a || b > n_tokens) { bad |= 1; return 0; }
+    if (b - a > max_len) { bad |= 2; return 0; }
+    return (uint32_t)(b - a) / (uint32_t)B;
+  };
+  // A CTA gives each warp R rounds of 32 consecutive requests (lane = request),
   // so that offsets are loaded and both outputs stored coalesced. Every offset
   // of the pass is loaded before any is used; the counts stay in registers
   // between the warp sums and the scans that write the outputs.
-  int64_t carry[NS] = {0, 0};
-  for (int64_t base = 0; base < n; base += (int64_t)blockDim.x * R) {
-    const int64_t seg = base + (int64_t)warp * 32 * R + lane;
+  const int64_t start = (int64_t)blockIdx.x * passes * kPrepPass;
+  int64_t before[NS] = {0, 0};  // this thread's share of the counts before the stretch
+#pragma unroll 8
+  for (int64_t r = tid; r < start; r += kPrepThreads) {
+    const uint32_t nb = blocks(__ldg(off + r), __ldg(off + r + 1));
+    before[0] += nb;
+    before[1] += (nb + 31) >> 5;
+  }
+  for (int64_t first = start; first < start + (int64_t)passes * kPrepPass && (first == start || first < n);
+       first += kPrepPass) {
+    const int64_t seg = first + (int64_t)warp * 32 * R + lane;
     int64_t a[R], b[R];
 #pragma unroll
     for (int i = 0; i < R; ++i) {
@@ -119,15 +155,7 @@ __global__ void __launch_bounds__(1024) k_prep(const int64_t* __restrict__ off, 
     }
     uint32_t nbv[R];
 #pragma unroll
-    for (int i = 0; i < R; ++i) {
-      uint32_t v = 0;
-      if (seg + 32 * i < n) {
-        if (a[i] < 0 || b[i] < a[i] || b[i] > n_tokens) bad |= 1;
-        else if (b[i] - a[i] > max_len) bad |= 2;
-        else v = (uint32_t)(b[i] - a[i]) / (uint32_t)B;
-      }
-      nbv[i] = v;
-    }
+    for (int i = 0; i < R; ++i) nbv[i] = seg + 32 * i < n ? blocks(a[i], b[i]) : 0;
     auto cnt = [&](int k, int i) -> int64_t { return k == 0 ? nbv[i] : (nbv[i] + 31) >> 5; };
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
@@ -136,24 +164,35 @@ __global__ void __launch_bounds__(1024) k_prep(const int64_t* __restrict__ off, 
       for (int i = 0; i < R; ++i) t += cnt(k, i);
 #pragma unroll
       for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(kFull, t, d);
-      if (lane == 0) warp_tot[k][warp] = t;
+      if (start > 0 && first == start) {
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) before[k] += __shfl_xor_sync(kFull, before[k], d);
+      }
+      if (lane == 0) {
+        warp_tot[k][warp] = t;
+        warp_before[k][warp] = before[k];
+      }
     }
     __syncthreads();
-    if (warp == 0) {
+    if (warp < NS) {  // warp k: scan k
+      const int k = warp;
+      const int64_t t = lane < nw ? warp_tot[k][lane] : 0;
+      int64_t carry = first > start ? pass_tot[k] : lane < nw ? warp_before[k][lane] : 0;
+      if (start > 0 && first == start) {
 #pragma unroll
-      for (int k = 0; k < NS; ++k) {
-        const int64_t t = lane < nw ? warp_tot[k][lane] : 0;
-        const int64_t ti = warp_incl_scan(t, lane);
-        if (lane < nw) warp_tot[k][lane] = ti - t;  // exclusive
-        if (lane == 31) pass_tot[k] = ti;
+        for (int d = 16; d > 0; d >>= 1) carry += __shfl_xor_sync(kFull, carry, d);
       }
+      __syncwarp();
+      const int64_t ti = warp_incl_scan(t, lane);
+      if (lane < nw) warp_tot[k][lane] = carry + ti - t;  // exclusive
+      if (lane == 31) pass_tot[k] = carry + ti;
     }
     __syncthreads();
     // both scans side by side, so that their shuffle chains overlap; rounds
     // past the last request are skipped (the test is warp-uniform)
     int64_t run[NS];
 #pragma unroll
-    for (int k = 0; k < NS; ++k) run[k] = carry[k] + warp_tot[k][warp];  // this warp's exclusive start
+    for (int k = 0; k < NS; ++k) run[k] = warp_tot[k][warp];  // this warp's exclusive start
 #pragma unroll
     for (int i = 0; i < R; ++i) {
       if (seg - lane + 32 * i >= n) break;
@@ -167,15 +206,13 @@ __global__ void __launch_bounds__(1024) k_prep(const int64_t* __restrict__ off, 
       run[0] += __shfl_sync(kFull, i0, 31);
       run[1] += __shfl_sync(kFull, i1, 31);
     }
-#pragma unroll
-    for (int k = 0; k < NS; ++k) carry[k] += pass_tot[k];
-    __syncthreads();  // warp_tot and pass_tot are rewritten by the next pass
+    __syncthreads();  // warp_tot is rewritten by the next pass
   }
   if (bad) atomicOr(&bad_all, bad);
   __syncthreads();
-  if (tid == 0) {
-    block_off[n] = carry[0];
-    if (chunk_off) chunk_off[n] = carry[1];
+  if (last && tid == 0) {
+    block_off[n] = pass_tot[0];
+    if (chunk_off) chunk_off[n] = pass_tot[1];
     const int ba = bad_all;
     *batch_ok = ba == 0;
     if (ba & 1) latch_error(status, SMETRIC_ERR_INVALID_ARG);
@@ -244,6 +281,23 @@ __device__ __forceinline__ void group_insert(uint64_t* __restrict__ groups, uint
     }
     s = (s + 1) & gmask;
   }
+}
+
+// The same by a whole warp (f warp-uniform), 32 points a step: two or three
+// dependent loads instead of up to fifteen.
+__device__ __forceinline__ int32_t find_request_warp(const int64_t* __restrict__ block_off, int32_t lo, int32_t n,
+                                                     int64_t f) {
+  const int lane = threadIdx.x & 31;
+  int32_t hi = n;
+  while (hi - lo > 1) {
+    const int32_t step = (hi - lo + 31) / 32;
+    const int64_t at = (int64_t)lo + (int64_t)lane * step;
+    const unsigned m = __ballot_sync(kFull, at < hi && __ldg(block_off + at) <= f);  // a prefix of the lanes, lane 0 in it
+    const int last = 31 - __clz(m);
+    hi = (int32_t)min((int64_t)hi, (int64_t)lo + (int64_t)(last + 1) * step);
+    lo += last * step;
+  }
+  return lo;
 }
 
 // Largest r in [lo, n) with block_off[r] <= f, given block_off[lo] <= f < block_off[n].
@@ -492,7 +546,7 @@ __global__ void __launch_bounds__(kTmaWarps * 32)
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;\n" : "=l"(policy));
   const int64_t token_bytes = 4 * n_tokens;
   const char* const tb = reinterpret_cast<const char*>(tokens);
-  int32_t r = find_request(chunk_off, 0, n, c_lo);  // warp-uniform
+  int32_t r = find_request_warp(chunk_off, 0, n, c_lo);
 
   // Start the copy of chunk c into stage s; returns this lane's first token
   // and sets its digest index and its request (`head` when the lane has the
@@ -817,8 +871,12 @@ __global__ void __launch_bounds__(256)
   const int64_t bo = __ldg(block_off + r), nb = __ldg(block_off + r + 1) - bo;
   int32_t l = r;
   int64_t sh = 0;
+  // the request's own leading digests, on their way while its leader is sought
+  uint64_t own[kGroupAhead];
+#pragma unroll
+  for (int u = 0; u < kGroupAhead; ++u) own[u] = 32 * u + lane < nb ? __ldg(D + bo + 32 * u + lane) : 0;
   if (nb > 0) {
-    const uint64_t key = chain_step(h_init, __ldg(D + bo));
+    const uint64_t key = chain_step(h_init, __shfl_sync(kFull, own[0], 0));
     const uint64_t s0 = key & gmask;
     for (uint64_t t = 0; t <= gmask; t += 32) {
       const uint64_t sl = (s0 + t + lane) & gmask;
@@ -837,11 +895,15 @@ __global__ void __launch_bounds__(256)
       sh = m;
       for (int64_t b = 0; b < m; b += 32 * kGroupAhead) {
         bool ne[kGroupAhead];
+        uint64_t other[kGroupAhead];
 #pragma unroll
         for (int u = 0; u < kGroupAhead; ++u) {
           const int64_t bb = b + 32 * u + lane;
-          ne[u] = bb < m && __ldg(D + bo + bb) != __ldg(D + lo + bb);
+          other[u] = bb < m ? __ldg(D + lo + bb) : 0;
+          if (b > 0) own[u] = bb < m ? __ldg(D + bo + bb) : 0;
         }
+#pragma unroll
+        for (int u = 0; u < kGroupAhead; ++u) ne[u] = b + 32 * u + lane < m && own[u] != other[u];
         int64_t first = -1;
 #pragma unroll
         for (int u = 0; u < kGroupAhead; ++u) {
@@ -2662,7 +2724,7 @@ int route_common(smetric_index* idx, const int32_t* d_tokens, int64_t n_tokens, 
   profile_begin(idx, s);
   // the policies' Eq. 1 arithmetic has its own limits on queues and lengths
   const bool eq1 = pol && (pol->on == kSession || pol->on == kColoc);
-  k_prep<<<1, 1024, 0, s>>>(d_offsets, n, n_tokens, c.block_size, d_load, PROBE ? c.num_instances : 0,
+  k_prep<<<prep_grid(n), kPrepThreads, 0, s>>>((int)prep_passes(n), d_offsets, n, n_tokens, c.block_size, d_load, PROBE ? c.num_instances : 0,
                             idx->block_off, idx->chunk_off, idx->batch_ok, idx->status,
                             eq1 ? SMETRIC_POLICY_MAX_QUEUED : SMETRIC_MAX_LOAD,
                             eq1 ? SMETRIC_POLICY_MAX_LEN : (int64_t)INT32_MAX, pol ? pol->est_hit : nullptr,
@@ -2941,7 +3003,7 @@ int commit_common(smetric_index* idx, const int64_t* d_offsets, int32_t n_reques
   if (!d_offsets || !d_instance || !d_block_hashes || (d_load && !d_local_hit)) return SMETRIC_ERR_INVALID_ARG;
   if (prep) {
     // block offsets of the batch (and the offsets' checks) into the index's scratch
-    k_prep<<<1, 1024, 0, s>>>(d_offsets, n_requests, c.max_batch_tokens, c.block_size, nullptr, 0, idx->block_off,
+    k_prep<<<prep_grid(n_requests), kPrepThreads, 0, s>>>((int)prep_passes(n_requests), d_offsets, n_requests, c.max_batch_tokens, c.block_size, nullptr, 0, idx->block_off,
                               nullptr, idx->batch_ok, idx->status, SMETRIC_MAX_LOAD, (int64_t)INT32_MAX, nullptr);
     idx->launches++;
     if ((rc = cuda_status(cudaGetLastError()))) return rc;
@@ -3349,7 +3411,7 @@ extern "C" int smetric_block_hashes_noalloc(const int32_t* d_tokens, int64_t n_t
   uint64_t* digest = scratch + kNaFlagWords + kNaOffWords;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
 
-  k_prep<<<1, 1024, 0, s>>>(d_offsets, n_requests, n_tokens, B, nullptr, 0, block_off, nullptr, ok, d_status,
+  k_prep<<<prep_grid(n_requests), kPrepThreads, 0, s>>>((int)prep_passes(n_requests), d_offsets, n_requests, n_tokens, B, nullptr, 0, block_off, nullptr, ok, d_status,
                             SMETRIC_MAX_LOAD, (int64_t)INT32_MAX, nullptr);
   if ((rc = cuda_status(cudaGetLastError()))) return rc;
   if (n_tokens / B > 0) {

@@ -7,6 +7,7 @@ import pytest
 torch = pytest.importorskip("torch")
 
 import oracle
+import paper_2607_08565_gb300 as pkg
 from gpu_util import T, assert_outputs_equal, gpu_hashes, gpu_route, make_index, populate_both
 from pins import GAMMA, M64, _py_mix64, py_mix64_inverse
 from synth.traces import pack
@@ -134,4 +135,31 @@ def test_sequential_stages_and_cost_widths(N, n):
         g = {k: v.cpu().numpy() for k, v in out.items()}
         assert_outputs_equal(g, o, fields=("instance", "local_hit", "global_hit", "session_key", "load_after"),
                              ctx=f"N={N} n={n} w={w}")
+    ix.close()
+
+
+@pytest.mark.parametrize("n", [8191, 8192, 8193, 16385, 1100000])
+def test_offsets_scanned_and_checked_in_stretches(n):
+    """Batches around the requests that one CTA of the offset scan takes (and one
+    past 128 times that): hashes equal the oracle's, and a bad offset or length
+    in any stretch makes the batch invalid."""
+    rng = np.random.default_rng(n)
+    B = 2
+    lens = rng.integers(0, 4, size=n)
+    off = np.zeros(n + 1, np.int64)
+    np.cumsum(lens, out=off[1:])
+    tok = _tokens(rng, off[-1])
+    ix = make_index(2, B, 1, max_req=n, max_tok=len(tok))
+    hb, sk = gpu_hashes(ix, tok, off)
+    o = oracle.OracleIndex(2).route_batch(B, 1, 0, tok, off, np.zeros(2, np.int64), 1, 4, 2, want_hashes=True,
+                                          n_threads=8)
+    assert np.array_equal(hb, o["block_hashes"]) and np.array_equal(sk, o["session_key"])
+    for at in (1, n // 2, n - 1):
+        bad = off.copy()
+        bad[at] = len(tok) + 1 if at % 2 else -1
+        d_sk = torch.full((n,), 5, dtype=torch.int64, device="cuda")
+        d_h = torch.zeros(max(1, len(tok) // B), dtype=torch.int64, device="cuda")
+        pkg.smetric_block_hashes(ix.handle, T(tok), len(tok), T(bad), n, d_sk, d_h, d_h.numel(), None)
+        assert ix.status() == pkg.SMETRIC_ERR_INVALID_ARG
+        assert not d_sk.any()
     ix.close()
