@@ -171,10 +171,9 @@ void free_all(smetric_index* x) {
   cudaFree(x->chunk_off);
   cudaFree(x->batch_ok);
   cudaFree(x->st_tokens);
-  cudaFree(x->st_offsets);
-  cudaFree(x->st_load);
-  cudaFree(x->st_out32);
-  cudaFree(x->st_sk);
+  cudaFree(x->st_in);
+  cudaFree(x->st_out);
+  cudaFreeHost(x->st_pin);
   for (auto& p : x->prof_pool)
     for (auto& e : p.ev) cudaEventDestroy(e);
   for (auto& p : x->prof_used)
@@ -238,10 +237,9 @@ int smetric_index_create(const smetric_index_config* cfg, smetric_index** out) {
   if (ok && (c.flags & SMETRIC_FLAG_HOST_STAGING)) {
     const size_t T = (size_t)(c.max_batch_tokens > 0 ? c.max_batch_tokens : 1);
     ok = cudaMalloc(&x->st_tokens, T * sizeof(int32_t)) == cudaSuccess &&
-         cudaMalloc(&x->st_offsets, (R + 1) * sizeof(int64_t)) == cudaSuccess &&
-         cudaMalloc(&x->st_load, (size_t)c.num_instances * sizeof(int64_t)) == cudaSuccess &&
-         cudaMalloc(&x->st_out32, (3 * R + 1) * sizeof(int32_t)) == cudaSuccess &&
-         cudaMalloc(&x->st_sk, (R + 1) * sizeof(uint64_t)) == cudaSuccess;
+         cudaMalloc(&x->st_in, ((size_t)c.num_instances + R + 1) * sizeof(int64_t)) == cudaSuccess &&
+         cudaMalloc(&x->st_out, (R + 1) * 20) == cudaSuccess &&
+         cudaMallocHost(&x->st_pin, kHostPin) == cudaSuccess;
   }
   if (ok && (c.flags & SMETRIC_FLAG_PIPELINE)) ok = pipeline_attach(x) == SMETRIC_OK;
   if (ok) ok = cudaMemset(x->table, 0, table_bytes) == cudaSuccess &&

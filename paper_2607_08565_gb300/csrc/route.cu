@@ -3258,23 +3258,52 @@ int smetric_route_batch_host(smetric_index* idx, const int32_t* h_tokens, int64_
       (n_tokens > 0 && !h_tokens))
     return SMETRIC_ERR_INVALID_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const size_t R = (size_t)n_requests;
+  const size_t R = (size_t)n_requests, N = (size_t)c.num_instances;
+  const bool small = n_requests <= kHostSmall;
+  int64_t* const d_load = idx->st_in;
+  int64_t* const d_offsets = idx->st_in + N;
+  uint64_t* const d_sk = idx->st_out;
+  int32_t* const o = reinterpret_cast<int32_t*>(idx->st_out + R);
+  unsigned char* const pin_out = idx->st_pin + kHostPinIn;
+  int32_t* const pin_status = reinterpret_cast<int32_t*>(pin_out + kHostPinOut);
   bool ok = true;
   if (n_tokens > 0)
     ok = ok && cudaMemcpyAsync(idx->st_tokens, h_tokens, (size_t)n_tokens * sizeof(int32_t),
                                cudaMemcpyHostToDevice, s) == cudaSuccess;
-  ok = ok && cudaMemcpyAsync(idx->st_offsets, h_offsets, (R + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s) == cudaSuccess;
-  ok = ok && cudaMemcpyAsync(idx->st_load, h_load, (size_t)c.num_instances * sizeof(int64_t),
-                             cudaMemcpyHostToDevice, s) == cudaSuccess;
-  if (!ok) return cuda_status(cudaErrorUnknown);
-  int32_t* o = idx->st_out32;
-  rc = smetric_route_batch(idx, idx->st_tokens, n_tokens, idx->st_offsets, n_requests, idx->st_load, w,
-                           o, o + R, o + 2 * R, idx->st_sk, nullptr, 0, stream);
-  if (rc) return rc;
+  if (small) {
+    int64_t* const pin_in = reinterpret_cast<int64_t*>(idx->st_pin);
+    memcpy(pin_in, h_load, N * sizeof(int64_t));
+    memcpy(pin_in + N, h_offsets, (R + 1) * sizeof(int64_t));
+    ok = ok && cudaMemcpyAsync(idx->st_in, pin_in, (N + R + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s) == cudaSuccess;
+  } else {
+    ok = ok && cudaMemcpyAsync(d_offsets, h_offsets, (R + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s) == cudaSuccess &&
+         cudaMemcpyAsync(d_load, h_load, N * sizeof(int64_t), cudaMemcpyHostToDevice, s) == cudaSuccess;
+  }
+  rc = ok ? smetric_route_batch(idx, idx->st_tokens, n_tokens, d_offsets, n_requests, d_load, w, o, o + R, o + 2 * R,
+                                d_sk, nullptr, 0, stream)
+          : cuda_status(cudaErrorUnknown);
+  if (rc) {
+    cudaStreamSynchronize(s);  // the pinned buffer may still be read
+    return rc;
+  }
+  if (small) {
+    // every output and the status, then one wait
+    ok = cudaMemcpyAsync(pin_out, idx->st_out, R * 20, cudaMemcpyDeviceToHost, s) == cudaSuccess &&
+         cudaMemcpyAsync(pin_status, idx->status, sizeof(int32_t), cudaMemcpyDeviceToHost, s) == cudaSuccess;
+    if (cudaStreamSynchronize(s) != cudaSuccess || !ok) return cuda_status(cudaErrorUnknown);
+    memcpy(h_session_key, pin_out, R * sizeof(uint64_t));
+    const unsigned char* const p = pin_out + R * sizeof(uint64_t);
+    memcpy(h_instance, p, R * sizeof(int32_t));
+    memcpy(h_local_hit, p + R * sizeof(int32_t), R * sizeof(int32_t));
+    memcpy(h_global_hit, p + 2 * R * sizeof(int32_t), R * sizeof(int32_t));
+    if (*pin_status != 0 && cudaMemset(idx->status, 0, sizeof(int32_t)) != cudaSuccess)
+      return cuda_status(cudaErrorUnknown);
+    return *pin_status;
+  }
   ok = cudaMemcpyAsync(h_instance, o, R * sizeof(int32_t), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
        cudaMemcpyAsync(h_local_hit, o + R, R * sizeof(int32_t), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
        cudaMemcpyAsync(h_global_hit, o + 2 * R, R * sizeof(int32_t), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
-       cudaMemcpyAsync(h_session_key, idx->st_sk, R * sizeof(uint64_t), cudaMemcpyDeviceToHost, s) == cudaSuccess;
+       cudaMemcpyAsync(h_session_key, d_sk, R * sizeof(uint64_t), cudaMemcpyDeviceToHost, s) == cudaSuccess;
   if (!ok) return cuda_status(cudaErrorUnknown);
   return smetric_status(idx, stream);
 }
