@@ -55,7 +55,11 @@ constexpr unsigned kFull = 0xffffffffu;
 
 constexpr int kChunk = 32;        // blocks per digest task (one per lane)
 constexpr int kDigestWarps = 8;   // most warps per digest CTA
-constexpr int kTmaWarps = 24;     // warps per TMA digest CTA (two CTAs per SM)
+// Warps per TMA digest CTA: as many rows as shared memory holds either way, two
+// CTAs an SM for B = 16 and 32, one for 64 (24 warps) and 128 (12 warps). The
+// largest box is 256 elements wide, so B = 256 stays with k_digest_any. Routes
+// of 2,466 requests of 17,144 tokens with B = 128: 79 us, 170 with k_digest_any.
+constexpr int tma_warps(int HB) { return HB <= 32 ? 24 : 12; }
 constexpr int kTmaStages = 1;     // copy stages per TMA digest warp
 constexpr int kMatchWarps = 8;    // warps per walk CTA
 constexpr int kGroupAhead = 8;    // 32-block rounds of digests a group warp compares at once
@@ -470,12 +474,13 @@ __global__ void __launch_bounds__(kDigestWarps * 32)
 // needs such a row, or whose blocks span two requests, is copied by its lanes
 // instead.
 
-constexpr int kMaxPhases = 16;  // 4B / 16 for B <= 64
 constexpr uint32_t kSpinLimit = 1u << 22;  // bounded mbarrier waits
 
+template <int HB>
 struct TokenMaps {
-  CUtensorMap map[kMaxPhases];
-  uint32_t rows[kMaxPhases];  // rows addressable through map k
+  static constexpr int kPhases = HB > 0 ? HB / 2 : 1;  // 4B / 16
+  CUtensorMap map[kPhases];
+  uint32_t rows[kPhases];  // rows addressable through map k
 };
 
 __device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t count) {
@@ -509,8 +514,8 @@ __device__ __forceinline__ void tma_rows(uint32_t dst, const CUtensorMap* map, i
 }
 
 template <int HB, int STAGES>
-__global__ void __launch_bounds__(kTmaWarps * 32)
-    k_digest_tma(const __grid_constant__ TokenMaps maps, const int32_t* __restrict__ tokens,
+__global__ void __launch_bounds__(tma_warps(HB) * 32)
+    k_digest_tma(const __grid_constant__ TokenMaps<HB> maps, const int32_t* __restrict__ tokens,
                  int64_t n_tokens, const int64_t* __restrict__ off, const int64_t* __restrict__ block_off,
                  const int64_t* __restrict__ chunk_off, int32_t n, uint64_t d_init, const int32_t* __restrict__ batch_ok,
                  uint64_t* __restrict__ digest, int32_t* status, uint64_t* __restrict__ groups, uint64_t gmask,
@@ -2449,7 +2454,9 @@ EncodeTiledFn tensor_map_encoder() {
 
 // One map per 16-byte phase k of a row start: base tokens + 16k, rows of
 // 4B+16 bytes at stride 4B, as many rows as fit inside the token buffer.
-bool make_token_maps(TokenMaps& m, const int32_t* tokens, int64_t n_tokens, int B) {
+template <int HB>
+bool make_token_maps(TokenMaps<HB>& m, const int32_t* tokens, int64_t n_tokens) {
+  constexpr int B = 2 * HB;
   EncodeTiledFn enc = tensor_map_encoder();
   if (!enc) return false;
   memset(&m, 0, sizeof(m));
@@ -2495,12 +2502,12 @@ int launch_digest(smetric_index* idx, const int32_t* d_tokens, int64_t n_tokens,
   // rows of 16*nch bytes: a block's 4B bytes start at most 12 bytes past a
   // 16-byte boundary
   const int nch = HB > 0 ? HB / 2 + 1 : (4 * B + 12 + 15) / 16;
-  if (HB > 0 && B / 4 <= kMaxPhases) {
-    static thread_local TokenMaps maps;
-    if (make_token_maps(maps, d_tokens, n_tokens, B)) {
-      auto kern = k_digest_tma<(HB > 0 ? HB : 2), kTmaStages>;
+  if constexpr (HB > 0) {
+    static thread_local TokenMaps<HB> maps;
+    if (make_token_maps<HB>(maps, d_tokens, n_tokens)) {
+      auto kern = k_digest_tma<HB, kTmaStages>;
       const size_t per_warp = (size_t)kTmaStages * kChunk * nch * 16 + 8 * kTmaStages;
-      const int warps = kTmaWarps;
+      const int warps = tma_warps(HB);
       const size_t smem = (size_t)warps * per_warp;
       if (idx->digest_occ == 0) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
@@ -2549,6 +2556,7 @@ int dispatch_digest(smetric_index* idx, const int32_t* d_tokens, int64_t n_token
     case 16: return launch_digest<8>(idx, d_tokens, n_tokens, d_offsets, n, s, group);
     case 32: return launch_digest<16>(idx, d_tokens, n_tokens, d_offsets, n, s, group);
     case 64: return launch_digest<32>(idx, d_tokens, n_tokens, d_offsets, n, s, group);
+    case 128: return launch_digest<64>(idx, d_tokens, n_tokens, d_offsets, n, s, group);
     default: return launch_digest<0>(idx, d_tokens, n_tokens, d_offsets, n, s, group);
   }
 }
