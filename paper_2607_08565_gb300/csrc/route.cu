@@ -55,11 +55,14 @@ constexpr unsigned kFull = 0xffffffffu;
 
 constexpr int kChunk = 32;        // blocks per digest task (one per lane)
 constexpr int kDigestWarps = 8;   // most warps per digest CTA
-// Warps per TMA digest CTA: as many rows as shared memory holds either way, two
-// CTAs an SM for B = 16 and 32, one for 64 (24 warps) and 128 (12 warps). The
-// largest box is 256 elements wide, so B = 256 stays with k_digest_any. Routes
-// of 2,466 requests of 17,144 tokens with B = 128: 79 us, 170 with k_digest_any.
-constexpr int tma_warps(int HB) { return HB <= 32 ? 24 : 12; }
+// Warps per TMA digest CTA, one CTA an SM: 32 for B = 16 and 32, then as many
+// rows as shared memory holds, 24 for B = 64 and 12 for 128. (The largest box is
+// 256 elements wide, so B = 256 stays with k_digest_any.) Measured, 205M tokens
+// with B = 32: 138 us; two CTAs of 24 warps 142.6, three of 16 145, one of 28
+// 144.6, two stages a warp 147 and more. 98M tokens with B = 16: 88 us, 90.6
+// with two CTAs of 24. Routes of 2,466 requests of 17,144 tokens with B = 128:
+// 79 us, 170 with k_digest_any.
+constexpr int tma_warps(int HB) { return HB <= 16 ? 32 : HB <= 32 ? 24 : 12; }
 constexpr int kTmaStages = 1;     // copy stages per TMA digest warp
 constexpr int kMatchWarps = 8;    // warps per walk CTA
 constexpr int kGroupAhead = 8;    // 32-block rounds of digests a group warp compares at once
