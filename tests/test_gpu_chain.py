@@ -109,6 +109,41 @@ def test_sentinel_in_the_middle_of_a_chain(at):
         ix.close()
 
 
+@pytest.mark.parametrize("more", [0, 1, 31, 33, 5000])
+@pytest.mark.parametrize("phase", [0, 1, 2, 3])
+def test_hashes_of_more_than_32_requests_an_sm(more, phase):
+    """Hash-only calls on both sides of 32 requests an SM, where a thread per
+    request takes over: lengths around its four blocks an access, hash buffers
+    in every 32-byte phase, a chain value of 0 and of 1 on the way."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n, B, S = 32 * sms + more, 2, 9
+    rng = np.random.default_rng(10 * more + phase)
+    reqs = [_tokens(rng, k) for k in np.minimum(rng.integers(0, 50, size=n), rng.integers(0, 50, size=n))]
+    reqs[7], reqs[n - 1] = _tokens(rng, 2 * 1300 + 1), _tokens(rng, 2 * 677)
+    for target in (0, 1):
+        head = _tokens(rng, 2 * (18 + target))
+        d = py_mix64_inverse(target) ^ ((int(oracle.block_hashes(head, 2, 0)[-1]) + GAMMA) & M64)
+        w = py_mix64_inverse(d) ^ _py_mix64(2)
+        block = np.array([w & 0xFFFFFFFF, w >> 32], dtype=np.uint32).view(np.int32)
+        reqs[100 + target] = np.concatenate([head, block, _tokens(rng, 41)])
+    tok, off = pack(reqs)
+    ix = make_index(4, B, S, max_req=n, max_tok=len(tok))
+    o = oracle.OracleIndex(4).route_batch(B, S, 0, tok, off, np.zeros(4, np.int64), 1, 4, 2, want_hashes=True,
+                                          n_threads=8)
+    nb = len(o["block_hashes"])
+    cap = len(tok) // B
+    buf = torch.full((cap + 8,), -1, dtype=torch.int64, device="cuda")
+    sk = torch.empty(n, dtype=torch.int64, device="cuda")
+    pkg.smetric_block_hashes(ix.handle, T(tok), len(tok), T(off), n, sk, buf[phase:], cap, None)
+    ix.check()
+    h = buf.cpu().numpy().view(np.uint64)
+    assert np.array_equal(h[phase:phase + nb], o["block_hashes"])
+    assert np.array_equal(sk.cpu().numpy().view(np.uint64), o["session_key"])
+    assert (h[:phase] == 2 ** 64 - 1).all() and (h[phase + nb:] == 2 ** 64 - 1).all()
+    assert {2, 3} <= set(h.tolist())
+    ix.close()
+
+
 @pytest.mark.parametrize("N", [1, 32, 33, 65, 128, 129, 256])
 @pytest.mark.parametrize("n", [1, 11, 12, 13, 37, 301])
 def test_sequential_stages_and_cost_widths(N, n):
