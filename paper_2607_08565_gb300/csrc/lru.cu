@@ -249,7 +249,10 @@ __global__ void __launch_bounds__(1024)
 
 // Thread per block f of the batch (request r, position b of n_r): into the
 // index, and its touch, whose position in a tier's list is the tier's count of
-// earlier requests' blocks plus n_r - 1 - b (deepest block first).
+// earlier requests' blocks plus n_r - 1 - b (deepest block first). The plan has
+// counted every block of a request that goes to an instance, so a block whose
+// hash is refused (below 2) has its places all the same: it leaves key 0 there,
+// which k_lru_flags passes over.
 __global__ void __launch_bounds__(256)
     k_lru_touch(uint8_t* tags, uint64_t* table, uint64_t n_buckets, int ew, const int64_t* __restrict__ block_off,
                 int32_t n, const int32_t* __restrict__ instance, const uint64_t* __restrict__ H,
@@ -264,6 +267,7 @@ __global__ void __launch_bounds__(256)
   int32_t r = 0;
   auto touch = [&](int t, int64_t q, uint64_t key) {
     touches[row(plan, nt, kTouchOff)[t] + q] = key;
+    if (key == 0) return;
     const uint32_t bit = filter_bit(key, row(plan, nt, kBitMask)[t]);
     atomicOr(filter + row(plan, nt, kBitOff)[t] + (bit >> 5), 1u << (bit & 31));
     const uint64_t e = set_put(set + 2 * row(plan, nt, kSetOff)[t], row(plan, nt, kSetMask)[t], key, (uint64_t)q + 1);
@@ -273,8 +277,11 @@ __global__ void __launch_bounds__(256)
        f += (int64_t)gridDim.x * blockDim.x) {
     r = request_of(block_off, r, n, f);
     const int32_t i = instance[r];
-    const uint64_t key = H[f];
-    if (!commit_block(tags, table, n_buckets, ew, N, key, i, global, status)) continue;
+    uint64_t key = H[f];
+    if (!commit_block(tags, table, n_buckets, ew, N, key, i, global, status)) {
+      if (i < 0 || i >= N) continue;  // no places
+      key = 0;
+    }
     const int64_t back = block_off[r + 1] - 1 - f;  // n_r - 1 - b
     if (local_capped) touch(i, req_off[r] + back, key);
     if (global_touch) touch(N, req_off[R + r] + back, key);
@@ -417,7 +424,7 @@ __global__ void __launch_bounds__(kLruThreads)
     for (int e = 0; e < kLruPer; ++e) {
       const uint32_t b = filter_bit(key[e], bmask);
       const bool hit = (__ldg(bits + (b >> 5)) >> (b & 31)) & 1u;
-      maybe |= (uint32_t)(hit && j0 + 32 * e < x.len + x.touch) << e;
+      maybe |= (uint32_t)(hit && key[e] != 0) << e;  // (0: past the tile's elements, or a refused touch)
     }
   }
 #pragma unroll
