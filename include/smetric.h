@@ -79,7 +79,7 @@ enum {
 #define SMETRIC_MAX_PROBE 65536
 
 /* smetric_index_config.flags */
-#define SMETRIC_FLAG_HOST_STAGING 1 /* allocate device staging buffers, and 60 KB of pinned host memory, for smetric_route_batch_host */
+#define SMETRIC_FLAG_HOST_STAGING 1 /* allocate device staging buffers, and 41 KB of pinned host memory, for smetric_route_batch_host */
 #define SMETRIC_FLAG_PIPELINE 2     /* allocate a second route scratch set for smetric_route_batches */
 
 typedef struct {

@@ -3362,28 +3362,20 @@ int smetric_route_batch_host(smetric_index* idx, const int32_t* h_tokens, int64_
   int64_t* const d_offsets = idx->st_in + N;
   uint64_t* const d_sk = idx->st_out;
   int32_t* const o = reinterpret_cast<int32_t*>(idx->st_out + R);
-  unsigned char* const pin_out = idx->st_pin + kHostPinIn;
+  unsigned char* const pin_out = idx->st_pin;
   int32_t* const pin_status = reinterpret_cast<int32_t*>(pin_out + kHostPinOut);
+  // The caller's arrays are read when the stream gets there: pinned ones may still be written by what is enqueued
+  // before this call.
   bool ok = true;
   if (n_tokens > 0)
     ok = ok && cudaMemcpyAsync(idx->st_tokens, h_tokens, (size_t)n_tokens * sizeof(int32_t),
                                cudaMemcpyHostToDevice, s) == cudaSuccess;
-  if (small) {
-    int64_t* const pin_in = reinterpret_cast<int64_t*>(idx->st_pin);
-    memcpy(pin_in, h_load, N * sizeof(int64_t));
-    memcpy(pin_in + N, h_offsets, (R + 1) * sizeof(int64_t));
-    ok = ok && cudaMemcpyAsync(idx->st_in, pin_in, (N + R + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s) == cudaSuccess;
-  } else {
-    ok = ok && cudaMemcpyAsync(d_offsets, h_offsets, (R + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s) == cudaSuccess &&
-         cudaMemcpyAsync(d_load, h_load, N * sizeof(int64_t), cudaMemcpyHostToDevice, s) == cudaSuccess;
-  }
-  rc = ok ? smetric_route_batch(idx, idx->st_tokens, n_tokens, d_offsets, n_requests, d_load, w, o, o + R, o + 2 * R,
-                                d_sk, nullptr, 0, stream)
-          : cuda_status(cudaErrorUnknown);
-  if (rc) {
-    cudaStreamSynchronize(s);  // the pinned buffer may still be read
-    return rc;
-  }
+  ok = ok && cudaMemcpyAsync(d_offsets, h_offsets, (R + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s) == cudaSuccess &&
+       cudaMemcpyAsync(d_load, h_load, N * sizeof(int64_t), cudaMemcpyHostToDevice, s) == cudaSuccess;
+  if (!ok) return cuda_status(cudaErrorUnknown);
+  rc = smetric_route_batch(idx, idx->st_tokens, n_tokens, d_offsets, n_requests, d_load, w, o, o + R, o + 2 * R,
+                           d_sk, nullptr, 0, stream);
+  if (rc) return rc;
   if (small) {
     // every output and the status, then one wait
     ok = cudaMemcpyAsync(pin_out, idx->st_out, R * 20, cudaMemcpyDeviceToHost, s) == cudaSuccess &&
