@@ -55,6 +55,10 @@ constexpr unsigned kFull = 0xffffffffu;
 
 constexpr int kChunk = 32;        // blocks per digest task (one per lane)
 constexpr int kDigestWarps = 8;   // most warps per digest CTA
+// Most shared memory of a digest CTA without tile copies. The limit on dynamic
+// shared memory belongs to the kernel, which every index (and the call without
+// one) shares: it is always set to this, never to what one block size needs.
+constexpr size_t kDigestSmem = 200 * 1024;
 // Warps per TMA digest CTA, one CTA an SM: 32 for B = 16 and 32, then as many
 // rows as shared memory holds, 24 for B = 64 and 12 for 128. (The largest box is
 // 256 elements wide, so B = 256 stays with k_digest_any.) Measured, 205M tokens
@@ -2610,12 +2614,12 @@ int launch_digest(smetric_index* idx, const int32_t* d_tokens, int64_t n_tokens,
     }
   }
   const size_t per_warp = (size_t)kChunk * nch * 16;
-  const int warps = (int)std::max<size_t>(1, std::min<size_t>(kDigestWarps, (200 * 1024) / per_warp));
+  const int warps = (int)std::max<size_t>(1, std::min<size_t>(kDigestWarps, kDigestSmem / per_warp));
   const size_t smem = (size_t)warps * per_warp;
   auto kern = HB > 0 ? k_digest<HB> : nullptr;
   const void* fn = HB > 0 ? (const void*)kern : (const void*)k_digest_any;
   if (idx->digest_occ == 0) {  // once per index: B, and so the plan, is fixed
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDigestSmem) != cudaSuccess)
       return cuda_status(cudaErrorInvalidValue);
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, warps * 32, smem) != cudaSuccess)
@@ -3482,11 +3486,11 @@ int na_digest(const int32_t* d_tokens, int64_t n_tokens, const int64_t* d_offset
   const int64_t max_chunks = (n_tokens / B + kChunk - 1) / kChunk;
   const int nch = HB > 0 ? HB / 2 + 1 : (4 * B + 12 + 15) / 16;
   const size_t per_warp = (size_t)kChunk * nch * 16;
-  const int warps = (int)std::max<size_t>(1, std::min<size_t>(kDigestWarps, (200 * 1024) / per_warp));
+  const int warps = (int)std::max<size_t>(1, std::min<size_t>(kDigestWarps, kDigestSmem / per_warp));
   const size_t smem = (size_t)warps * per_warp;
   const void* fn = HB > 0 ? (const void*)k_digest<(HB > 0 ? HB : 2)> : (const void*)k_digest_any;
   int occ = 0;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDigestSmem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, warps * 32, smem) != cudaSuccess)
     return cuda_status(cudaErrorInvalidValue);
   const int64_t want = (max_chunks + warps - 1) / warps;
