@@ -242,7 +242,7 @@ int smetric_index_create(const smetric_index_config* cfg, smetric_index** out) {
          cudaMallocHost(&x->st_pin, kHostPin) == cudaSuccess;
   }
   if (ok && (c.flags & SMETRIC_FLAG_PIPELINE)) ok = pipeline_attach(x) == SMETRIC_OK;
-  if (ok) ok = cudaMemset(x->table, 0, table_bytes) == cudaSuccess &&
+  if (ok) ok = kernel_limits(x) && cudaMemset(x->table, 0, table_bytes) == cudaSuccess &&
                cudaMemset(x->tags, 0, tag_bytes) == cudaSuccess &&
                cudaMemset(x->status, 0, sizeof(int32_t)) == cudaSuccess &&
                cudaMemset(x->groups, 0, 2 * x->group_slots * sizeof(uint64_t)) == cudaSuccess &&

@@ -139,6 +139,9 @@ __device__ __forceinline__ int64_t next_pow2(int64_t v) {
 // A key's bit in a filter; the sets use the low bits.
 __device__ __forceinline__ uint32_t filter_bit(uint64_t key, int64_t mask) { return (uint32_t)(key >> 32) & (uint32_t)mask; }
 
+// Its shared memory: running totals, and a round's totals per warp, of N + 1 tiers.
+constexpr size_t plan_smem(int N) { return (size_t)33 * (N + 1) * sizeof(int64_t); }
+
 // One CTA: checks and drain, then rounds of 1,024 requests, 32 to a warp.
 // Within a warp, the lanes routed to the same instance (__match_any_sync) sum
 // the blocks of their lower lanes; the warps' totals per instance are scanned
@@ -579,10 +582,7 @@ int lru_commit(smetric_index* idx, const int64_t* d_offsets, const int32_t* d_in
   const int64_t R = idx->cfg.max_batch_requests;
   const int64_t max_blocks = idx->cfg.max_batch_tokens / idx->cfg.block_size;
   int rc;
-  const size_t smem = (size_t)33 * (N + 1) * sizeof(int64_t);
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(k_lru_plan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return cuda_status(cudaErrorInvalidValue);
+  const size_t smem = plan_smem(N);
   const int64_t want = (max_blocks + 255) / 256;
   const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)idx->num_sms * 8));
   const uint64_t* ring = L->ring[L->cur];
@@ -623,6 +623,10 @@ int smetric_index_set_lru(smetric_index* idx, int64_t local_cap, int64_t global_
   if (cudaDeviceSynchronize() != cudaSuccess) return cuda_status(cudaErrorUnknown);
   lru_free(idx);
   if (local_cap == 0 && global_cap == 0) return SMETRIC_OK;
+  // the plan kernel's limit is every index's: the most that any N takes
+  if (cudaFuncSetAttribute(k_lru_plan, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)plan_smem(SMETRIC_MAX_INSTANCES)) != cudaSuccess)
+    return cuda_status(cudaErrorInvalidValue);
   const int N = idx->cfg.num_instances, nt = N + 1;
   const int64_t R = idx->cfg.max_batch_requests;
   const int64_t max_blocks = idx->cfg.max_batch_tokens / idx->cfg.block_size;

@@ -759,7 +759,8 @@ constexpr int kCpMaxLanes = 32 * kCpMaxChainWarps;
 // lanes' rows of one slot an odd number of 16-byte units, so that a chain
 // warp's 16-byte accesses meet no bank conflict.
 constexpr int kCpRow = 272;
-constexpr int kCpMaxSlots = 8;       // 8 with one or two chain warps, 4 with more (139 KB of ring at most)
+constexpr int kCpMaxSlots = 8;       // 8 with one or two chain warps, 4 with more
+constexpr size_t kCpMaxRing = (size_t)kCpMaxLanes * (kCpMaxSlots / 2) * kCpRow;  // 139,264 bytes, and with two warps too
 constexpr int kCpRound = 512;        // requests a CTA takes at a time
 
 __device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
@@ -2660,9 +2661,23 @@ int launch_chain_probe(ChainArgs a, int num_sms, cudaStream_t s, bool pdl) {
   a.chain_warps = (int)std::max<int64_t>(1, std::min<int64_t>(kCpMaxChainWarps, (per_cta + 31) / 32));
   a.slots = a.chain_warps <= 2 ? kCpMaxSlots : kCpMaxSlots / 2;
   const size_t smem = (size_t)32 * a.chain_warps * a.slots * kCpRow;
-  if (cudaFuncSetAttribute(k_chain_probe<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return cuda_status(cudaErrorInvalidValue);
   return launch_k(k_chain_probe<W>, dim3((unsigned)grid), dim3(cp_warps(W) * 32), smem, s, pdl, a);
+}
+
+// The limits on dynamic shared memory of the chain kernel and of the sequential
+// decisions. A limit belongs to the kernel and not to the index or the call, so
+// it is set to the most that any call takes, once per index (the call without an
+// index sets it itself), and never lowered: a call on another index and thread
+// may come between any two of this one's.
+template <int W>
+bool chain_limit() {
+  return cudaFuncSetAttribute(k_chain_probe<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCpMaxRing) == cudaSuccess;
+}
+template <int T>
+constexpr size_t seq_smem() { return (size_t)kSeqStages * kSeqWarps * 32 * T * sizeof(SeqEntry); }
+template <int T>
+bool seq_limit() {
+  return cudaFuncSetAttribute(k_seq<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)seq_smem<T>()) == cudaSuccess;
 }
 
 // The hash-only calls' chain.
@@ -2904,6 +2919,17 @@ int route_policy(smetric_index* idx, int mode, const int32_t* d_tokens, int64_t 
 // ---------------------------------------------------------------------------
 
 namespace smetric {
+
+// Shared-memory limits of the kernels that index x's calls launch with more than
+// 48 KB (the digest's is set on its first call, the LRU's by smetric_index_set_lru).
+bool kernel_limits(const smetric_index* x) {
+  const bool chain = x->W == 1   ? chain_limit<1>()
+                     : x->W == 2 ? chain_limit<2>()
+                     : x->W == 3 ? chain_limit<3>()
+                     : x->W == 4 ? chain_limit<4>()
+                                 : chain_limit<5>();
+  return chain && chain_limit<0>() && seq_limit<1>() && seq_limit<2>() && seq_limit<4>() && seq_limit<8>();
+}
 
 // The second route scratch set of an index created with SMETRIC_FLAG_PIPELINE:
 // the same buffers, with the same sizes, as the index's own set.
@@ -3160,17 +3186,16 @@ int smetric_route_batch_sequential(smetric_index* idx, const int32_t* d_tokens, 
   if (rc || n_requests == 0) return rc;
   idx->launches++;
   const int N = idx->cfg.num_instances;
-  auto launch = [&](auto kern, int T) {
-    const size_t smem = (size_t)kSeqStages * kSeqWarps * 32 * T * sizeof(SeqEntry);
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return cuda_status(cudaErrorInvalidValue);
+  auto launch = [&](auto kern, size_t smem) {
     kern<<<1, kSeqBlock * 32, smem, s>>>(N, idx->cfg.block_size, d_offsets, n_requests, d_load, w.w_load,
                                                w.w_miss, w.w_glob, idx->summ, idx->batch_ok, d_instance, d_local_hit,
                                                d_global_hit, d_load_after, idx->status);
     return cuda_status(cudaGetLastError());
   };
-  return N <= 32 ? launch(k_seq<1>, 1) : N <= 64 ? launch(k_seq<2>, 2) : N <= 128 ? launch(k_seq<4>, 4) : launch(k_seq<8>, 8);
+  return N <= 32    ? launch(k_seq<1>, seq_smem<1>())
+         : N <= 64  ? launch(k_seq<2>, seq_smem<2>())
+         : N <= 128 ? launch(k_seq<4>, seq_smem<4>())
+                    : launch(k_seq<8>, seq_smem<8>());
 }
 
 int smetric_route_batch_baseline(smetric_index* idx, const int32_t* d_tokens, int64_t n_tokens,
@@ -3557,5 +3582,6 @@ extern "C" int smetric_block_hashes_noalloc(const int32_t* d_tokens, int64_t n_t
   a.hashes = d_block_hashes;
   a.sk_out = d_session_key;
   a.status = d_status;
+  if (!chain_limit<0>()) return cuda_status(cudaErrorInvalidValue);
   return launch_chain(a, num_sms, s, false);
 }

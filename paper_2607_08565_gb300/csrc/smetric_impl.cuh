@@ -183,6 +183,8 @@ struct smetric_index {
 namespace smetric {
 // Returns SMETRIC_OK if the index is usable from the current device.
 int check_device(const smetric_index* idx);
+// Sets the shared-memory limits of the index's kernels; false on a CUDA error.
+bool kernel_limits(const smetric_index* idx);
 // Maps a CUDA error to SMETRIC_ERR_CUDA (clearing the sticky-free error state).
 int cuda_status(cudaError_t e);
 // Inserts a routed batch's block hashes into its chosen instances' local tiers

@@ -1,6 +1,8 @@
 """Several indexes in one process: kernels that they share serve each of them,
 whatever the others' block sizes and batch sizes are."""
 
+import threading
+
 import numpy as np
 import pytest
 
@@ -35,3 +37,41 @@ def test_block_sizes_in_turn(large, small):
         assert np.array_equal(got, want[B]), B
     first.close()
     second.close()
+
+
+@pytest.mark.parametrize("commit,shapes", [(False, ((7, 2000), (7, 6080))), (True, ((190, 5), (256, 5)))])
+def test_threads_on_indexes_of_their_own(commit, shapes):
+    """Eight threads, each with an index and a stream; their batches want different amounts of shared memory."""
+    B, rounds, L = 2, 5000, pkg.lib()
+    failed = []
+
+    def work(N, n):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            ix = make_index(N, B, 1, max_req=n, max_tok=n * B)
+            off = T(np.arange(n + 1, dtype=np.int64) * B)
+            tok, load, out = T(np.zeros(n * B, np.int32)), T(np.zeros(N, np.int64)), T(np.zeros((3, n), np.int32))
+            h = T(np.arange(2, n + 2))
+            if commit:
+                ix.set_lru(8)
+            a, s, w = out.data_ptr(), stream.cuda_stream, pkg.smetric_weights(1, 4, 2)
+            stream.synchronize()
+            for i in range(rounds):
+                if commit:
+                    rc = L.smetric_index_commit_batch(ix.handle, off.data_ptr(), n, a, a + 4 * n, h.data_ptr(), 0, None, s)
+                else:
+                    rc = L.smetric_route_batch(ix.handle, tok.data_ptr(), n * B, off.data_ptr(), n, load.data_ptr(), w,
+                                               a, a + 4 * n, a + 8 * n, h.data_ptr(), None, 0, s)
+                failed.extend([rc] if rc else [])
+                if i % 200 == 0:
+                    stream.synchronize()
+            ix.check()
+            done.append(n)
+
+    done = []
+    threads = [threading.Thread(target=work, args=shapes[k % 2]) for k in range(8)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed and len(done) == 8
