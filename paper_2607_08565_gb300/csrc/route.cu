@@ -2576,6 +2576,13 @@ uint64_t group_slots_for(int32_t n) {
   return g;
 }
 
+// Empties the group table of a call of n requests whose last kernel, which does
+// that, could not be launched.
+void empty_groups(smetric_index* idx, int32_t n, cudaStream_t s) {
+  (void)cudaMemsetAsync(idx->groups, 0, 2 * sizeof(uint64_t) * group_slots_for(n), s);
+  (void)cudaGetLastError();  // (the call returns the first error)
+}
+
 // The digest kernel for the index's block size; with `group` it also puts
 // each request's first-block hash into the group table.
 template <int HB>
@@ -2859,8 +2866,10 @@ int route_common(smetric_index* idx, const int32_t* d_tokens, int64_t n_tokens, 
   if (PROBE) {
     const WalkPolicy off_pol = {};
     if ((rc = dispatch_match(idx, d_offsets, n, d_load, w, inst, lhit, ghit, hashes, sk,
-                             n_tokens / c.block_size, pol ? *pol : off_pol, s, ov)))
+                             n_tokens / c.block_size, pol ? *pol : off_pol, s, ov))) {
+      empty_groups(idx, n, s);  // the walk that would have emptied the table was not launched
       return rc;
+    }
   } else {
     ChainArgs a = chain_args(idx, n, sk);
     a.hashes = hashes;
@@ -3354,8 +3363,10 @@ int smetric_link_sessions(smetric_index* idx, const int32_t* d_tokens, int64_t n
       (rc = launch_k(k_link_chase, g, t, 0, s, true, n_requests, ok, (const int32_t*)d_parent, d_session, st)) ||
       (rc = launch_k(k_link_heads, dim3((unsigned)std::min<int64_t>(1 + ((int64_t)gmask + 1024) / 1024, idx->num_sms)),
                      dim3(1024), 0, s, true, n_requests, ok, d_parent, d_session, vecs, (int64_t)(gmask + 1),
-                     (const LinkState*)st)))
+                     (const LinkState*)st))) {
+    empty_groups(idx, n_requests, s);
     return rc;
+  }
   return SMETRIC_OK;
 }
 
