@@ -27,12 +27,12 @@
 //                 its touch (deepest block first) into its tiers' touch lists,
 //                 the batch's (tier, key) -> last touch sets (noting the
 //                 touch's entry there) and their filters.
-//   k_lru_flags   CTA per tile of 1,024 records-then-touches of one tier: a
+//   k_lru_flags   CTAs over tiles of 1,024 records-then-touches of one tier: a
 //                 bit for whether each survives the rewrite, and the tile's
 //                 count.
 //   k_lru_scan    one CTA: exclusive scan of the tile counts; per tier its
 //                 surviving count and the excess over its cap.
-//   k_lru_write   CTA per tile: each survivor's rank in its tier; the first
+//   k_lru_write   CTAs over the tiles: each survivor's rank in its tier; the first
 //                 `excess` go to the list of evicted keys, the rest to the
 //                 other buffer.
 //   k_lru_evict   thread per evicted key: remove_tier, which gives a slot back
@@ -68,6 +68,13 @@ constexpr int kLruPer = 4;                           // rounds of 32 consecutive
 // the lookups; 4,096 a tile left those to a few dozen CTAs (31 us instead of 24
 // for the flags kernel at 190k touches of one tier).
 constexpr int64_t kLruTile = kLruThreads * kLruPer;
+// CTAs an SM of the two kernels over the tiles, at most. The caps say how many
+// tiles there may be, the tiers' lengths how many there are: a CTA for each that
+// may be made a commit of 3,200 blocks on 272M capped blocks take 324 us (these
+// limits 75), and 95 on 48M (66). Full tiers want many CTAs, so that the tiles
+// with the lookups spread: 717k blocks a commit on 48M records take 872 us with
+// 192 of the flags kernel, 882 with 64, 870 with a CTA a tile.
+constexpr int kFlagCtas = 192, kWriteCtas = 64;
 constexpr int kLruTileWords = (int)(kLruTile / 32);  // flag words of a tile
 constexpr int64_t kMaxCap = 1LL << 40;
 
@@ -396,14 +403,11 @@ __global__ void __launch_bounds__(1024)
   }
 }
 
-__global__ void __launch_bounds__(kLruThreads)
-    k_lru_flags(const int64_t* __restrict__ plan, int nt, const uint64_t* __restrict__ ring,
-                const uint64_t* __restrict__ touches, const uint32_t* __restrict__ where,
-                const uint64_t* __restrict__ set, const uint32_t* __restrict__ filter, uint32_t* __restrict__ keep,
-                int64_t* __restrict__ tile_cnt) {
-  pdl_enter();
-  const int64_t k = blockIdx.x;
-  if (k >= row(plan, nt, kTile0)[nt]) return;
+// Flags and count of tile k, by one CTA.
+__device__ __forceinline__ void flag_tile(int64_t k, const int64_t* __restrict__ plan, int nt, const uint64_t* __restrict__ ring,
+                                          const uint64_t* __restrict__ touches, const uint32_t* __restrict__ where,
+                                          const uint64_t* __restrict__ set, const uint32_t* __restrict__ filter, uint32_t* __restrict__ keep,
+                                          int64_t* __restrict__ tile_cnt) {
   const LruTile x = tile_of(plan, nt, k, ring, touches);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t j0 = x.j0 + (int64_t)w * 32 * kLruPer + lane;
@@ -492,36 +496,54 @@ __global__ void __launch_bounds__(kLruThreads)
   }
 }
 
+// LOOP: a CTA takes every gridDim.x-th tile, with fewer CTAs than there may be
+// tiles. (Without it the loop's two registers would cost 0.3 % of a commit.)
+template <bool LOOP>
+__global__ void __launch_bounds__(kLruThreads)
+    k_lru_flags(const int64_t* __restrict__ plan, int nt, const uint64_t* __restrict__ ring,
+                const uint64_t* __restrict__ touches, const uint32_t* __restrict__ where,
+                const uint64_t* __restrict__ set, const uint32_t* __restrict__ filter, uint32_t* __restrict__ keep,
+                int64_t* __restrict__ tile_cnt) {
+  pdl_enter();
+  const int64_t total = row(plan, nt, kTile0)[nt];
+  for (int64_t k = blockIdx.x; k < total; k += gridDim.x) {
+    flag_tile(k, plan, nt, ring, touches, where, set, filter, keep, tile_cnt);
+    if (!LOOP) return;
+    __syncthreads();  // the next tile takes the shared arrays
+  }
+}
+
 __global__ void __launch_bounds__(kLruThreads)
     k_lru_write(const int64_t* __restrict__ plan, int nt, const uint64_t* __restrict__ ring,
                 uint64_t* __restrict__ next, const uint64_t* __restrict__ touches, const uint32_t* __restrict__ keep,
                 const int64_t* __restrict__ tile_off, uint64_t* __restrict__ evicted) {
   pdl_enter();
   const int64_t* tile0 = row(plan, nt, kTile0);
-  const int64_t k = blockIdx.x;
+  const int64_t total = tile0[nt];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (k >= tile0[nt]) return;
-  const LruTile x = tile_of(plan, nt, k, ring, touches);
-  // lane e < kLruPer has the warp's flag word e; survivors of the CTA's earlier warps
-  const uint32_t* const words = keep + k * kLruTileWords;
-  const uint32_t mine = lane < kLruPer ? words[w * kLruPer + lane] : 0;
-  int before = 0;
-  for (int u = lane; u < w * kLruPer; u += 32) before += __popc(words[u]);
-  before = __reduce_add_sync(0xffffffffu, before);
-  int64_t rank = tile_off[k] - tile_off[tile0[x.t]] + before;
-  const int64_t ex = row(plan, nt, kExcess)[x.t];
-  const int64_t j0 = x.j0 + (int64_t)w * 32 * kLruPer + lane;
-  uint64_t* const out = next + row(plan, nt, kRingOff)[x.t] - ex;
-  uint64_t* const gone = evicted + row(plan, nt, kEvictOff)[x.t];
-  uint64_t key[kLruPer];
+  for (int64_t k = blockIdx.x; k < total; k += gridDim.x) {
+    const LruTile x = tile_of(plan, nt, k, ring, touches);
+    // lane e < kLruPer has the warp's flag word e; survivors of the CTA's earlier warps
+    const uint32_t* const words = keep + k * kLruTileWords;
+    const uint32_t mine = lane < kLruPer ? words[w * kLruPer + lane] : 0;
+    int before = 0;
+    for (int u = lane; u < w * kLruPer; u += 32) before += __popc(words[u]);
+    before = __reduce_add_sync(0xffffffffu, before);
+    int64_t rank = tile_off[k] - tile_off[tile0[x.t]] + before;
+    const int64_t ex = row(plan, nt, kExcess)[x.t];
+    const int64_t j0 = x.j0 + (int64_t)w * 32 * kLruPer + lane;
+    uint64_t* const out = next + row(plan, nt, kRingOff)[x.t] - ex;
+    uint64_t* const gone = evicted + row(plan, nt, kEvictOff)[x.t];
+    uint64_t key[kLruPer];
 #pragma unroll
-  for (int e = 0; e < kLruPer; ++e) key[e] = element(x, j0 + 32 * e);
+    for (int e = 0; e < kLruPer; ++e) key[e] = element(x, j0 + 32 * e);
 #pragma unroll
-  for (int e = 0; e < kLruPer; ++e) {
-    const uint32_t m = __shfl_sync(0xffffffffu, mine, e);
-    const int64_t at = rank + __popc(m & ((1u << lane) - 1));
-    if ((m >> lane) & 1u) (at >= ex ? out : gone)[at] = key[e];
-    rank += __popc(m);
+    for (int e = 0; e < kLruPer; ++e) {
+      const uint32_t m = __shfl_sync(0xffffffffu, mine, e);
+      const int64_t at = rank + __popc(m & ((1u << lane) - 1));
+      if ((m >> lane) & 1u) (at >= ex ? out : gone)[at] = key[e];
+      rank += __popc(m);
+    }
   }
 }
 
@@ -585,6 +607,9 @@ int lru_commit(smetric_index* idx, const int64_t* d_offsets, const int32_t* d_in
   const size_t smem = plan_smem(N);
   const int64_t want = (max_blocks + 255) / 256;
   const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)idx->num_sms * 8));
+  const int64_t tiles = L->max_tiles;
+  const unsigned fgrid = (unsigned)std::min<int64_t>(tiles, (int64_t)idx->num_sms * kFlagCtas);
+  const unsigned wgrid = (unsigned)std::min<int64_t>(tiles, (int64_t)idx->num_sms * kWriteCtas);
   const uint64_t* ring = L->ring[L->cur];
   uint64_t* next = L->ring[L->cur ^ 1];
   if ((rc = launch_k(k_lru_plan, dim3(1), dim3(1024), smem, s, true, d_offsets, (const int64_t*)idx->block_off, n,
@@ -594,13 +619,13 @@ int lru_commit(smetric_index* idx, const int64_t* d_offsets, const int32_t* d_in
                      (const int64_t*)idx->block_off, n, d_instance, d_hashes, (const int32_t*)idx->batch_ok, N, global,
                      local_capped, global_touch, (const int64_t*)L->plan, (const int64_t*)L->req_off, R, L->touches,
                      L->where, L->set, L->filter, idx->status)) ||
-      (rc = launch_k(k_lru_flags, dim3((unsigned)L->max_tiles), dim3(kLruThreads), 0, s, true,
+      (rc = launch_k(tiles > fgrid ? k_lru_flags<true> : k_lru_flags<false>, dim3(fgrid), dim3(kLruThreads), 0, s, true,
                      (const int64_t*)L->plan, nt, ring,
                      (const uint64_t*)L->touches, (const uint32_t*)L->where, (const uint64_t*)L->set,
                      (const uint32_t*)L->filter, L->keep, L->tile_cnt)) ||
       (rc = launch_k(k_lru_scan, dim3(1), dim3(1024), 0, s, true, L->plan, nt, (const int64_t*)L->tile_cnt,
                      L->tile_off)) ||
-      (rc = launch_k(k_lru_write, dim3((unsigned)L->max_tiles), dim3(kLruThreads), 0, s, true,
+      (rc = launch_k(k_lru_write, dim3(wgrid), dim3(kLruThreads), 0, s, true,
                      (const int64_t*)L->plan, nt, ring, next, (const uint64_t*)L->touches, (const uint32_t*)L->keep,
                      (const int64_t*)L->tile_off, L->evicted)) ||
       (rc = launch_k(k_lru_evict, dim3(grid), dim3(256), 0, s, true, L->plan, nt, (const uint64_t*)L->evicted, L->set,

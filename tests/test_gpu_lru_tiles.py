@@ -47,3 +47,37 @@ def test_lru_tiles_and_plan_rounds(N, local_cap, global_cap):
             got = keys[(m[:, bit >> 6] >> np.uint64(bit & 63)) & np.uint64(1) == 1]
             assert set(got.tolist()) == set(ol.stamp[t]), (step, t)
     ix.close()
+
+
+@pytest.mark.parametrize("n,per,cap", [(7, 30, 1000), (4000, 1000, 30_500_000)])
+def test_more_tiles_than_ctas(n, per, cap):
+    """Commits on one tier, at the largest with more tiles than the kernels have CTAs; a key's stamp is that of
+    its last touch, and the tier keeps the `cap` largest (on the small case the LRU oracle says the same)."""
+    N, B, K = 2, 2, 9
+    ix = make_index(N, B, 1, cap=2 * K * n * per, max_req=n, max_tok=n * per * B)
+    ix.set_lru(cap)
+    off = torch.arange(n + 1, device="cuda") * (per * B)
+    who = torch.zeros(n, dtype=torch.int32, device="cuda")
+    key_of = lambda i: (i + 1) * -7046029254386353131  # noqa: E731  (odd: another key for every i)
+    ol = oracle.OracleLRU(N, local_cap=cap)
+    stamp = torch.zeros(K * n * per, dtype=torch.int64, device="cuda")
+    late = (torch.arange(n * per, device="cuda") // per + 1) * per - torch.arange(n * per, device="cuda") % per  # by request, then deepest first
+    for k in range(K):
+        first = k * n * per
+        i = torch.arange(first, first + n * per, device="cuda")
+        if k % 2:  # half of it was there before, some of that evicted since
+            i[: n * per // 2] = i[: n * per // 2] * 3 // 5
+        h = key_of(i)
+        ix.commit_batch(off, dict(instance=who, local_hit=torch.zeros_like(who), block_hashes=h))
+        stamp.scatter_reduce_(0, i, late + first, "amax")
+        if n < 100:
+            ol.commit(np.full(n, per), who.cpu().numpy(), h.cpu().numpy().view(np.uint64), also_global=False)
+    ix.check()
+    assert ix.lru_sizes().tolist() == [min(cap, int((stamp > 0).sum())), 0, 0]
+    least = torch.sort(stamp, descending=True).values[cap - 1]
+    held = (ix.lookup(key_of(torch.arange(K * n * per, device="cuda"))).view(torch.int64)[:, 0] & 1) == 1
+    assert torch.equal(held, (stamp >= least) & (stamp > 0))
+    if n < 100:
+        keys = key_of(torch.arange(K * n * per, device="cuda"))[held].cpu().numpy().view(np.uint64)
+        assert set(keys.tolist()) == set(ol.stamp[0])
+    ix.close()
