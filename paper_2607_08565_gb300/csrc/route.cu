@@ -474,20 +474,24 @@ __global__ void __launch_bounds__(kDigestWarps * 32)
 //
 // For B % 4 == 0, block j of a request starts 4B*j bytes after block 0, so the
 // rows a_j = (4*first token of block j) & ~15 of one request form a strided
-// 2D region: rows of 4B+16 bytes at stride 4B. A 2D tensor map per 16-byte
-// phase k (base = tokens + 16k) with row stride 4B and row length 4B+16 lets
-// one TMA tile load of 32 rows bring a whole chunk into the padded layout.
-// Rows past the end of the map are zero-filled by the TMA unit; a chunk that
-// needs such a row, or whose blocks span two requests, is copied by its lanes
-// instead.
+// 2D region: rows of 4B+16 bytes at stride 4B. A 2D tensor map with row stride
+// 4B lets one TMA tile load of 32 rows bring a whole chunk into the padded
+// layout. Up to B = 64 there is a map per 16-byte phase k of a_0 (base = tokens +
+// 16k, rows of 4B+16 bytes); for B = 128 one map with rows of 8B bytes serves
+// every phase, at column 16k. (With 32 maps a call took 2.2 us more on the host;
+// with one map at B = 32 the digest of 205M tokens took 1.4 us more.)
+// Every row of a map lies inside the token buffer; rows past its end are
+// zero-filled by the TMA unit, and a chunk that needs such a row is copied by its
+// lanes instead.
 
 constexpr uint32_t kSpinLimit = 1u << 22;  // bounded mbarrier waits
 
 template <int HB>
 struct TokenMaps {
   static constexpr int kPhases = HB > 0 ? HB / 2 : 1;  // 4B / 16
-  CUtensorMap map[kPhases];
-  uint32_t rows[kPhases];  // rows addressable through map k
+  static constexpr int kMaps = kPhases <= 16 ? kPhases : 1;
+  CUtensorMap map[kMaps];
+  uint32_t rows[kMaps];  // rows addressable through map k
 };
 
 __device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t count) {
@@ -511,11 +515,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity) {
     if (mbar_try_wait(mbar, parity)) return true;
   return false;
 }
-__device__ __forceinline__ void tma_rows(uint32_t dst, const CUtensorMap* map, int32_t y, uint32_t mbar,
+__device__ __forceinline__ void tma_rows(uint32_t dst, const CUtensorMap* map, int32_t x, int32_t y, uint32_t mbar,
                                          uint64_t policy) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
-      " [%0], [%1, {%2, %3}], [%4], %5;\n" ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(0),
+      " [%0], [%1, {%2, %3}], [%4], %5;\n" ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x),
       "r"(y), "r"(mbar), "l"(policy)
       : "memory");
 }
@@ -575,7 +579,9 @@ __global__ void __launch_bounds__(tma_warps(HB) * 32)
     head = b == 0;
     const int nv = (int)min((int64_t)kChunk, nbr - (b - lane));
     const int64_t a0 = (4 * __shfl_sync(kFull, tok0, 0)) & ~(int64_t)15;
-    const int k = (int)((a0 % (4 * B)) >> 4);
+    const int phase16 = (int)((a0 % (4 * B)) >> 4);
+    const int k = TokenMaps<HB>::kMaps > 1 ? phase16 : 0;
+    const int x = TokenMaps<HB>::kMaps > 1 ? 0 : 4 * phase16;  // first token of the row: a multiple of 16 bytes
     const int64_t y0 = a0 / (4 * B);
     unsigned char* const st = stages + (size_t)s * STAGE;
     const uint32_t mbar = mbar0 + 8u * (uint32_t)s;
@@ -583,7 +589,7 @@ __global__ void __launch_bounds__(tma_warps(HB) * 32)
       if (lane == 0) {
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         mbar_arrive_expect_tx(mbar, STAGE);
-        tma_rows(smem_u32(st), &maps.map[k], (int32_t)y0, mbar, policy);
+        tma_rows(smem_u32(st), &maps.map[k], x, (int32_t)y0, mbar, policy);
       }
     } else {
       // lanes copy their own rows; the stage's barrier completes on lane 0's
@@ -2541,21 +2547,20 @@ EncodeTiledFn tensor_map_encoder() {
   return fn;
 }
 
-// One map per 16-byte phase k of a row start: base tokens + 16k, rows of
-// 4B+16 bytes at stride 4B, as many rows as fit inside the token buffer.
+// The maps of a token buffer: base tokens + 16k, as many rows as fit inside it.
 template <int HB>
 bool make_token_maps(TokenMaps<HB>& m, const int32_t* tokens, int64_t n_tokens) {
-  constexpr int B = 2 * HB;
+  constexpr int B = 2 * HB, maps = TokenMaps<HB>::kMaps, width = maps > 1 ? B + 4 : 2 * B;
   EncodeTiledFn enc = tensor_map_encoder();
   if (!enc) return false;
   memset(&m, 0, sizeof(m));
-  const int64_t bytes = 4 * n_tokens, row = 4 * B + 16, stride = 4 * B;
-  for (int k = 0; k < B / 4; ++k) {
+  const int64_t bytes = 4 * n_tokens, row = 4 * width, stride = 4 * B;
+  for (int k = 0; k < maps; ++k) {
     const int64_t base = 16 * k;
     if (bytes < base + row) continue;  // rows[k] = 0: chunks fall back to lane copies
     int64_t rows = (bytes - base - row) / stride + 1;
     if (rows > INT32_MAX) rows = INT32_MAX;
-    const cuuint64_t dims[2] = {(cuuint64_t)(B + 4), (cuuint64_t)rows};
+    const cuuint64_t dims[2] = {(cuuint64_t)width, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)stride};
     const cuuint32_t box[2] = {(cuuint32_t)(B + 4), (cuuint32_t)kChunk};
     const cuuint32_t es[2] = {1, 1};
