@@ -1102,12 +1102,18 @@ __global__ void __launch_bounds__(cp_warps(W) * 32, 1) k_chain_probe(const Chain
     const int32_t m = min(kCpRound, m_all - g0);
     const int act = min(m, lanes);  // lanes in use
     // ---- the round's requests; with more than one per lane, longest first
-    int32_t k = -1, r = 0, nb = 0;  // this thread's request: its place in lane order, index and full blocks
+    int32_t k = -1;  // this thread's request: its place in lane order
+    ChainReq x = {};
     if (threadIdx.x < (unsigned)m) {
       k = (int32_t)threadIdx.x;
-      r = dealt ? s_mine[g0 + k] : (int32_t)blockIdx.x + (g0 + k) * stride;
-      nb = (int32_t)(__ldg(a.block_off + r + 1) - __ldg(a.block_off + r));
-      s_len0[k] = nb;
+      x.req = dealt ? s_mine[g0 + k] : (int32_t)blockIdx.x + (g0 + k) * stride;
+      x.bo = __ldg(a.block_off + x.req);
+      x.nb = (int32_t)(__ldg(a.block_off + x.req + 1) - x.bo);
+      if (W > 0) {
+        x.cb = __ldg(a.chunk_off + x.req);
+        x.share = __ldg(a.share + x.req);
+      }
+      s_len0[k] = x.nb;
     }
     if (threadIdx.x < kCpMaxLanes) s_len[threadIdx.x] = 0;
     if (threadIdx.x < kCpMaxChainWarps) s_most[threadIdx.x] = s_pos[threadIdx.x] = 0;
@@ -1132,7 +1138,7 @@ __global__ void __launch_bounds__(cp_warps(W) * 32, 1) k_chain_probe(const Chain
         int32_t rank = 0;
         for (int32_t i = 0; i < m; ++i) {
           const int32_t v = s_len0[i];
-          rank += v > nb || (v == nb && i < (int32_t)threadIdx.x);
+          rank += v > x.nb || (v == x.nb && i < (int32_t)threadIdx.x);
         }
         const int32_t pass = rank / lanes, at = rank % lanes;
         k = pass * lanes + ((pass & 1) ? at : min(lanes, m - pass * lanes) - 1 - at);
@@ -1140,17 +1146,9 @@ __global__ void __launch_bounds__(cp_warps(W) * 32, 1) k_chain_probe(const Chain
     }
     __syncthreads();
     if (k >= 0) {
-      ChainReq x = {};
-      x.bo = __ldg(a.block_off + r);
-      x.nb = nb;
-      x.req = r;
-      if (W > 0) {
-        x.cb = __ldg(a.chunk_off + r);
-        x.share = __ldg(a.share + r);
-        s_dead[k] = INT32_MAX;
-      }
+      if (W > 0) s_dead[k] = INT32_MAX;
       s_rq[k] = x;
-      if (nb == 0) a.sk_out[r] = 0;
+      if (x.nb == 0) a.sk_out[x.req] = 0;
     }
     __syncthreads();
     if (threadIdx.x < (unsigned)act) {
