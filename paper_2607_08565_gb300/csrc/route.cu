@@ -757,7 +757,9 @@ __device__ __forceinline__ void probe_one(const uint8_t* __restrict__ tags, cons
 // Chunk q of request r is its blocks 32q .. 32q + 31; the chunk ANDs the walk reads are kept per such
 // request-aligned chunk, at index chunk_off[r] + q.
 constexpr int kCpWarps = 32;
-constexpr int kHashWarps = 24;       // without an index; 8,192 prompts of 750 blocks: 109 us, with 32 warps 113, with 16 120
+// Without an index (32 requests an SM at most: one chain warp). 4,096 prompts of
+// 750 blocks: 45.6 us, with 24 warps 48.7, with 32 49.7; 1,024 prompts 40.2, 41.2, 41.2.
+constexpr int kHashWarps = 16;
 __host__ __device__ constexpr int cp_warps(int W) { return W == 0 ? kHashWarps : kCpWarps; }
 constexpr int kCpMaxChainWarps = 4;  // warps 0 .. 3, one per scheduler
 constexpr int kCpMaxLanes = 32 * kCpMaxChainWarps;
