@@ -3,9 +3,9 @@
 // every request of the batch routed against one snapshot of index and load).
 //
 // Kernels per batch, in stream order:
-//   k_prep        one CTA: validates offsets and loads; scans the per-request
-//                 full-block counts into block_off and the 32-block chunk
-//                 counts into chunk_off.
+//   k_prep        a CTA per 8,192 requests (up to 128): validates offsets and
+//                 loads; scans the per-request full-block counts into block_off
+//                 and the 32-block chunk counts into chunk_off.
 //   k_digest_tma  HBM-bound block digests d_b: chunk q of request r is its
 //                 blocks 32q..32q+31, one 2D TMA tile of 32 overlapping rows
 //                 (each block's bytes rounded out to 16-byte boundaries); a
@@ -67,7 +67,11 @@ constexpr size_t kDigestSmem = 200 * 1024;
 // with two CTAs of 24. Routes of 2,466 requests of 17,144 tokens with B = 128:
 // 79 us, 170 with k_digest_any.
 constexpr int tma_warps(int HB) { return HB <= 16 ? 32 : HB <= 32 ? 24 : 12; }
-constexpr int kTmaStages = 1;     // copy stages per TMA digest warp
+// Copy stages per TMA digest warp. The kernel is written for any number: for one
+// alone, without its loops over stages, ptxas took 32 to 36 registers instead of
+// 40, and routes 274 us instead of 269 (8,192 requests, B = 32) and 399 instead
+// of 289 (4,099 requests, N = 256, B = 16).
+constexpr int kTmaStages = 1;
 constexpr int kMatchWarps = 8;    // warps per walk CTA
 constexpr int kGroupAhead = 8;    // 32-block rounds of digests a group warp compares at once
 
@@ -294,9 +298,9 @@ __device__ __forceinline__ void group_insert(uint64_t* __restrict__ groups, uint
   }
 }
 
-// The same by a whole warp (f warp-uniform), 32 points a step: two or three
+// request_of by a whole warp (f warp-uniform), 32 points a step: two or three
 // dependent loads instead of up to fifteen.
-__device__ __forceinline__ int32_t find_request_warp(const int64_t* __restrict__ block_off, int32_t lo, int32_t n,
+__device__ __forceinline__ int32_t request_of_warp(const int64_t* __restrict__ block_off, int32_t lo, int32_t n,
                                                      int64_t f) {
   const int lane = threadIdx.x & 31;
   int32_t hi = n;
@@ -307,17 +311,6 @@ __device__ __forceinline__ int32_t find_request_warp(const int64_t* __restrict__
     const int last = 31 - __clz(m);
     hi = (int32_t)min((int64_t)hi, (int64_t)lo + (int64_t)(last + 1) * step);
     lo += last * step;
-  }
-  return lo;
-}
-
-// Largest r in [lo, n) with block_off[r] <= f, given block_off[lo] <= f < block_off[n].
-__device__ __forceinline__ int32_t find_request(const int64_t* __restrict__ block_off, int32_t lo,
-                                                int32_t n, int64_t f) {
-  int32_t hi = n;
-  while (hi - lo > 1) {
-    const int32_t mid = (lo + hi) >> 1;
-    if (__ldg(block_off + mid) <= f) lo = mid; else hi = mid;
   }
   return lo;
 }
@@ -393,7 +386,7 @@ __global__ void __launch_bounds__(kDigestWarps * 32)
   const int64_t token_bytes = 4 * n_tokens;
   const char* const tb = reinterpret_cast<const char*>(tokens);
 
-  int32_t r = find_request(block_off, 0, n, min(c_lo * kChunk + lane, total - 1));
+  int32_t r = request_of(block_off, 0, n, min(c_lo * kChunk + lane, total - 1));
 
   struct Chunk {
     int64_t tok0;  // this lane's first token
@@ -410,7 +403,7 @@ __global__ void __launch_bounds__(kDigestWarps * 32)
     ch.head = false;
     ch.req = r;
     if (ch.valid) {
-      if (__ldg(block_off + r + 1) <= f) r = find_request(block_off, r + 1, n, f);
+      if (__ldg(block_off + r + 1) <= f) r = request_of(block_off, r + 1, n, f);
       ch.tok0 = __ldg(off + r) + (f - __ldg(block_off + r)) * B;
       ch.head = f == __ldg(block_off + r);
       ch.req = r;
@@ -562,14 +555,14 @@ __global__ void __launch_bounds__(tma_warps(HB) * 32)
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;\n" : "=l"(policy));
   const int64_t token_bytes = 4 * n_tokens;
   const char* const tb = reinterpret_cast<const char*>(tokens);
-  int32_t r = find_request_warp(chunk_off, 0, n, c_lo);
+  int32_t r = request_of_warp(chunk_off, 0, n, c_lo);
 
   // Start the copy of chunk c into stage s; returns this lane's first token
   // and sets its digest index and its request (`head` when the lane has the
   // request's block 0, whose digest also gives the request's group key).
   auto issue = [&](int64_t c, int s, bool& valid, int64_t& gidx, int32_t& req, bool& head) -> int64_t {
     for (int i = 0; i < 4 && __ldg(chunk_off + r + 1) <= c; ++i) ++r;  // usually a step or two
-    if (__ldg(chunk_off + r + 1) <= c) r = find_request(chunk_off, r + 1, n, c);
+    if (__ldg(chunk_off + r + 1) <= c) r = request_of(chunk_off, r + 1, n, c);
     const int64_t bo = __ldg(block_off + r), nbr = __ldg(block_off + r + 1) - bo;
     const int64_t b = (c - __ldg(chunk_off + r)) * kChunk + lane;  // block of request r
     valid = b < nbr;
@@ -670,11 +663,11 @@ __global__ void __launch_bounds__(kDigestWarps * 32)
   uint4* const row = dsm + ((size_t)warp * kChunk + lane) * nch;
   const int64_t token_bytes = 4 * n_tokens;
   const char* const tb = reinterpret_cast<const char*>(tokens);
-  int32_t r = find_request(block_off, 0, n, min(c_lo * kChunk + lane, total - 1));
+  int32_t r = request_of(block_off, 0, n, min(c_lo * kChunk + lane, total - 1));
   for (int64_t c = c_lo; c < c_hi; ++c) {
     const int64_t f = c * kChunk + lane;
     if (f >= total) continue;
-    if (__ldg(block_off + r + 1) <= f) r = find_request(block_off, r + 1, n, f);
+    if (__ldg(block_off + r + 1) <= f) r = request_of(block_off, r + 1, n, f);
     const int64_t tok0 = __ldg(off + r) + (f - __ldg(block_off + r)) * B;
     const int64_t a = (4 * tok0) & ~(int64_t)15;
     for (int i = 0; i < nch; ++i) row[i] = load_piece(tb, a + 16 * i, token_bytes - (a + 16 * i));
@@ -1954,8 +1947,7 @@ __global__ void __launch_bounds__(kSeqBlock * 32)
       const int slot = st % kSeqStages;
       const Row x = rows[u];
       load_row((int64_t)(st + kSeqAhead) * kSeqWarps + warp, rows[u]);
-      // (the deciding warp shares a scheduler with some of these: 32-bit
-      // factors, all within their limits, and the smallest rest as its decision)
+      // (32-bit factors, all within their limits; the smallest rest as the deciding warp finds its minimum)
       uint64_t rest[T];
       uint32_t mh = 0xffffffffu, ml = 0xffffffffu;
       const uint32_t L = (uint32_t)x.L;
@@ -2715,8 +2707,7 @@ ChainArgs chain_args(const smetric_index* idx, int32_t n, uint64_t* sk) {
 template <int W>
 int launch_match(smetric_index* idx, const int64_t* d_offsets, int32_t n, const int64_t* d_load,
                  smetric_weights w, int32_t* inst, int32_t* lhit, int32_t* ghit, uint64_t* hashes,
-                 uint64_t* sk, int64_t max_blocks, const WalkPolicy& pol, cudaStream_t s,
-                 const Overlap* ov) {
+                 uint64_t* sk, const WalkPolicy& pol, cudaStream_t s, const Overlap* ov) {
   const cudaEvent_t after_chain = ov ? ov->after_chain : nullptr;
   const int N = idx->cfg.num_instances;
   int rc;
@@ -2728,28 +2719,26 @@ int launch_match(smetric_index* idx, const int64_t* d_offsets, int32_t n, const 
                      (n + idx->num_sms - 1) / idx->num_sms <= kCpRound;
   // one byte a request, in the scratch words k_link_sessions uses for its keys
   uint8_t* const flags = reinterpret_cast<uint8_t*>(idx->sk_tmp);
-  {
-    idx->launches++;
-    if ((rc = launch_k(k_lead, dim3((unsigned)((n + 7) / 8)), dim3(256), 0, s, !idx->profiling,
-                       (const int64_t*)idx->block_off, n, (const int32_t*)idx->batch_ok, (const uint64_t*)idx->digest,
-                       mix64(idx->cfg.hash_seed + kGamma), (const uint64_t*)idx->groups, group_slots_for(n) - 1, defer,
-                       idx->lead, idx->share, flags)))
-      return rc;
-    ChainArgs a = chain_args(idx, n, sk);
-    a.chunk_off = idx->chunk_off;
-    a.hashes = hashes ? hashes : defer ? idx->hashes : nullptr;
-    a.share = idx->share;
-    a.active = flags;
-    a.deal = defer;
-    a.tags = idx->tags;
-    a.table = idx->table;
-    a.n_buckets = idx->n_buckets;
-    a.masks = idx->masks;
-    a.chunk_and = idx->chunk_and;
-    idx->launches++;
-    if ((rc = launch_chain_probe<W>(a, idx->num_sms, s, !idx->profiling))) return rc;
-    if (after_chain && cudaEventRecord(after_chain, s) != cudaSuccess) return cuda_status(cudaErrorUnknown);
-  }
+  idx->launches++;
+  if ((rc = launch_k(k_lead, dim3((unsigned)((n + 7) / 8)), dim3(256), 0, s, !idx->profiling,
+                     (const int64_t*)idx->block_off, n, (const int32_t*)idx->batch_ok, (const uint64_t*)idx->digest,
+                     mix64(idx->cfg.hash_seed + kGamma), (const uint64_t*)idx->groups, group_slots_for(n) - 1, defer,
+                     idx->lead, idx->share, flags)))
+    return rc;
+  ChainArgs chain = chain_args(idx, n, sk);
+  chain.chunk_off = idx->chunk_off;
+  chain.hashes = hashes ? hashes : defer ? idx->hashes : nullptr;
+  chain.share = idx->share;
+  chain.active = flags;
+  chain.deal = defer;
+  chain.tags = idx->tags;
+  chain.table = idx->table;
+  chain.n_buckets = idx->n_buckets;
+  chain.masks = idx->masks;
+  chain.chunk_and = idx->chunk_and;
+  idx->launches++;
+  if ((rc = launch_chain_probe<W>(chain, idx->num_sms, s, !idx->profiling))) return rc;
+  if (after_chain && cudaEventRecord(after_chain, s) != cudaSuccess) return cuda_status(cudaErrorUnknown);
   profile_mark(idx, kChainProbe, s);
   const int64_t want = ((int64_t)n + kMatchWarps - 1) / kMatchWarps;
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)idx->num_sms * 8));
@@ -2798,14 +2787,13 @@ int launch_match(smetric_index* idx, const int64_t* d_offsets, int32_t n, const 
 
 int dispatch_match(smetric_index* idx, const int64_t* d_offsets, int32_t n, const int64_t* d_load,
                    smetric_weights w, int32_t* inst, int32_t* lhit, int32_t* ghit, uint64_t* hashes,
-                   uint64_t* sk, int64_t max_blocks, const WalkPolicy& pol, cudaStream_t s,
-                   const Overlap* ov) {
+                   uint64_t* sk, const WalkPolicy& pol, cudaStream_t s, const Overlap* ov) {
   switch (idx->W) {
-    case 1: return launch_match<1>(idx, d_offsets, n, d_load, w, inst, lhit, ghit, hashes, sk, max_blocks, pol, s, ov);
-    case 2: return launch_match<2>(idx, d_offsets, n, d_load, w, inst, lhit, ghit, hashes, sk, max_blocks, pol, s, ov);
-    case 3: return launch_match<3>(idx, d_offsets, n, d_load, w, inst, lhit, ghit, hashes, sk, max_blocks, pol, s, ov);
-    case 4: return launch_match<4>(idx, d_offsets, n, d_load, w, inst, lhit, ghit, hashes, sk, max_blocks, pol, s, ov);
-    case 5: return launch_match<5>(idx, d_offsets, n, d_load, w, inst, lhit, ghit, hashes, sk, max_blocks, pol, s, ov);
+    case 1: return launch_match<1>(idx, d_offsets, n, d_load, w, inst, lhit, ghit, hashes, sk, pol, s, ov);
+    case 2: return launch_match<2>(idx, d_offsets, n, d_load, w, inst, lhit, ghit, hashes, sk, pol, s, ov);
+    case 3: return launch_match<3>(idx, d_offsets, n, d_load, w, inst, lhit, ghit, hashes, sk, pol, s, ov);
+    case 4: return launch_match<4>(idx, d_offsets, n, d_load, w, inst, lhit, ghit, hashes, sk, pol, s, ov);
+    case 5: return launch_match<5>(idx, d_offsets, n, d_load, w, inst, lhit, ghit, hashes, sk, pol, s, ov);
     default: return SMETRIC_ERR_INVALID_ARG;
   }
 }
@@ -2870,8 +2858,7 @@ int route_common(smetric_index* idx, const int32_t* d_tokens, int64_t n_tokens, 
   profile_mark(idx, kDigest, s);
   if (PROBE) {
     const WalkPolicy off_pol = {};
-    if ((rc = dispatch_match(idx, d_offsets, n, d_load, w, inst, lhit, ghit, hashes, sk,
-                             n_tokens / c.block_size, pol ? *pol : off_pol, s, ov))) {
+    if ((rc = dispatch_match(idx, d_offsets, n, d_load, w, inst, lhit, ghit, hashes, sk, pol ? *pol : off_pol, s, ov))) {
       empty_groups(idx, n, s);  // the walk that would have emptied the table was not launched
       return rc;
     }
