@@ -470,9 +470,12 @@ __global__ void __launch_bounds__(kDigestWarps * 32)
 // 2D region: rows of 4B+16 bytes at stride 4B. A 2D tensor map with row stride
 // 4B lets one TMA tile load of 32 rows bring a whole chunk into the padded
 // layout. Up to B = 64 there is a map per 16-byte phase k of a_0 (base = tokens +
-// 16k, rows of 4B+16 bytes); for B = 128 one map with rows of 8B bytes serves
-// every phase, at column 16k. (With 32 maps a call took 2.2 us more on the host;
-// with one map at B = 32 the digest of 205M tokens took 1.4 us more.)
+// 16k, rows of 4B+16 bytes). For B = 128, rows of 8B bytes serve every phase, at
+// column 16k: one map from the buffer's start, and one whose rows end with the
+// buffer, for the chunk that the first one's last rows do not reach. (With 32
+// maps a call took 2.2 us more on the host; without the second, batches of 235
+// requests 1 us more, for their last chunk's lane copies; with such maps at B =
+// 32 the digest of 205M tokens 1.4 us more.)
 // Every row of a map lies inside the token buffer; rows past its end are
 // zero-filled by the TMA unit, and a chunk that needs such a row is copied by its
 // lanes instead.
@@ -482,9 +485,11 @@ constexpr uint32_t kSpinLimit = 1u << 22;  // bounded mbarrier waits
 template <int HB>
 struct TokenMaps {
   static constexpr int kPhases = HB > 0 ? HB / 2 : 1;  // 4B / 16
-  static constexpr int kMaps = kPhases <= 16 ? kPhases : 1;
+  static constexpr bool kWide = kPhases > 16;  // two maps for every phase
+  static constexpr int kMaps = kWide ? 2 : kPhases;
   CUtensorMap map[kMaps];
   uint32_t rows[kMaps];  // rows addressable through map k
+  uint32_t base[kMaps];  // its first byte in the token buffer
 };
 
 __device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t count) {
@@ -572,10 +577,18 @@ __global__ void __launch_bounds__(tma_warps(HB) * 32)
     head = b == 0;
     const int nv = (int)min((int64_t)kChunk, nbr - (b - lane));
     const int64_t a0 = (4 * __shfl_sync(kFull, tok0, 0)) & ~(int64_t)15;
-    const int phase16 = (int)((a0 % (4 * B)) >> 4);
-    const int k = TokenMaps<HB>::kMaps > 1 ? phase16 : 0;
-    const int x = TokenMaps<HB>::kMaps > 1 ? 0 : 4 * phase16;  // first token of the row: a multiple of 16 bytes
-    const int64_t y0 = a0 / (4 * B);
+    int k = (int)((a0 % (4 * B)) >> 4), x = 0;  // map, and column (in tokens, a multiple of 16 bytes)
+    int64_t y0 = a0 / (4 * B);
+    if constexpr (TokenMaps<HB>::kWide) {
+      x = 4 * k;
+      k = 0;
+      if (y0 + nv > (int64_t)maps.rows[0] && a0 >= (int64_t)maps.base[1]) {
+        const uint64_t e = (uint64_t)a0 - maps.base[1];
+        k = 1;
+        x = (int)((uint32_t)e % (4 * B)) >> 2;
+        y0 = (int64_t)(e / (4 * B));
+      }
+    }
     unsigned char* const st = stages + (size_t)s * STAGE;
     const uint32_t mbar = mbar0 + 8u * (uint32_t)s;
     if (y0 + nv <= (int64_t)maps.rows[k]) {
@@ -2539,16 +2552,18 @@ EncodeTiledFn tensor_map_encoder() {
   return fn;
 }
 
-// The maps of a token buffer: base tokens + 16k, as many rows as fit inside it.
+// The maps of a token buffer: as many rows as fit inside it from each map's base.
 template <int HB>
 bool make_token_maps(TokenMaps<HB>& m, const int32_t* tokens, int64_t n_tokens) {
-  constexpr int B = 2 * HB, maps = TokenMaps<HB>::kMaps, width = maps > 1 ? B + 4 : 2 * B;
+  using Maps = TokenMaps<HB>;
+  constexpr int B = 2 * HB, width = Maps::kWide ? 2 * B : B + 4;
   EncodeTiledFn enc = tensor_map_encoder();
   if (!enc) return false;
   memset(&m, 0, sizeof(m));
   const int64_t bytes = 4 * n_tokens, row = 4 * width, stride = 4 * B;
-  for (int k = 0; k < maps; ++k) {
-    const int64_t base = 16 * k;
+  for (int k = 0; k < Maps::kMaps; ++k) {
+    const int64_t base = !Maps::kWide ? 16 * k : k == 0 || bytes < row ? 0 : (bytes - row) % stride & ~(int64_t)15;
+    m.base[k] = (uint32_t)base;
     if (bytes < base + row) continue;  // rows[k] = 0: chunks fall back to lane copies
     int64_t rows = (bytes - base - row) / stride + 1;
     if (rows > INT32_MAX) rows = INT32_MAX;
