@@ -38,11 +38,12 @@
  *   - Calls are stream-ordered: inserts, evictions and routes enqueued on one
  *     stream see each other's effects in enqueue order. Calls on one index
  *     share that index's scratch, so they must not run concurrently on
- *     different streams.
+ *     different streams. Calls on different indexes may, from any threads.
  *   - Host-detectable errors return immediately with nothing enqueued.
  *     Device-detectable errors (bad offsets, out-of-range tiers or loads, a
  *     full table) are latched in the index and reported by smetric_status.
- *   - Nothing here allocates device memory except smetric_index_create.
+ *   - Nothing here allocates device memory except smetric_index_create and
+ *     smetric_index_set_lru.
  */
 #ifndef SMETRIC_H
 #define SMETRIC_H
@@ -481,9 +482,9 @@ int smetric_block_hashes_noalloc(const int32_t* d_tokens, int64_t n_tokens, cons
                                  uint64_t hash_seed, uint64_t* d_session_key, uint64_t* d_block_hashes,
                                  int64_t hashes_cap, int32_t* d_status, smetric_stream_t stream);
 
-/* smetric_route_batch from host buffers: copies tokens, offsets and load to
- * the index's staging buffers (the index must have been created with
- * SMETRIC_FLAG_HOST_STAGING), routes, copies the four outputs back and waits
+/* smetric_route_batch from host buffers: copies tokens, offsets and load, in
+ * stream order, to the index's staging buffers (the index must have been created
+ * with SMETRIC_FLAG_HOST_STAGING), routes, copies the four outputs back and waits
  * for the stream. Returns the call's status including any error the device
  * latched, which it clears. */
 int smetric_route_batch_host(smetric_index* idx, const int32_t* h_tokens, int64_t n_tokens,
