@@ -172,7 +172,6 @@ void free_all(smetric_index* x) {
   cudaFree(x->batch_ok);
   cudaFree(x->st_tokens);
   cudaFree(x->st_in);
-  cudaFree(x->st_out);
   cudaFreeHost(x->st_pin);
   for (auto& p : x->prof_pool)
     for (auto& e : p.ev) cudaEventDestroy(e);
@@ -216,11 +215,12 @@ int smetric_index_create(const smetric_index_config* cfg, smetric_index** out) {
   const size_t tag_bytes = (size_t)x->n_buckets * kBucket;
   const size_t max_blocks = (size_t)(c.max_batch_tokens / c.block_size);
   const size_t R = (size_t)c.max_batch_requests;
+  const bool staging = (c.flags & SMETRIC_FLAG_HOST_STAGING) != 0;
   x->group_slots = 64;
   while (x->group_slots < 2 * (uint64_t)R) x->group_slots <<= 1;
   bool ok = cudaMalloc(&x->table, table_bytes) == cudaSuccess &&
             cudaMalloc(&x->tags, tag_bytes) == cudaSuccess &&
-            cudaMalloc(&x->status, sizeof(int32_t)) == cudaSuccess &&
+            cudaMalloc(&x->status, kStatusBytes + (staging ? (R + 1) * 20 : 0)) == cudaSuccess &&
             cudaMalloc(&x->block_off, (R + 1) * sizeof(int64_t)) == cudaSuccess &&
             cudaMalloc(&x->digest, (max_blocks > 0 ? max_blocks : 1) * sizeof(uint64_t)) == cudaSuccess &&
             cudaMalloc(&x->hashes, (max_blocks > 0 ? max_blocks : 1) * sizeof(uint64_t)) == cudaSuccess &&
@@ -234,12 +234,12 @@ int smetric_index_create(const smetric_index_config* cfg, smetric_index** out) {
             cudaMalloc(&x->summ, (R > 0 ? R : 1) * ((size_t)c.num_instances + 1) * sizeof(int32_t)) == cudaSuccess &&
             cudaMalloc(&x->batch_ok, sizeof(int32_t)) == cudaSuccess;
   if (ok) x->share = x->lead + (R + 1);
-  if (ok && (c.flags & SMETRIC_FLAG_HOST_STAGING)) {
+  if (ok && staging) {
     const size_t T = (size_t)(c.max_batch_tokens > 0 ? c.max_batch_tokens : 1);
     ok = cudaMalloc(&x->st_tokens, T * sizeof(int32_t)) == cudaSuccess &&
          cudaMalloc(&x->st_in, ((size_t)c.num_instances + R + 1) * sizeof(int64_t)) == cudaSuccess &&
-         cudaMalloc(&x->st_out, (R + 1) * 20) == cudaSuccess &&
          cudaMallocHost(&x->st_pin, kHostPin) == cudaSuccess;
+    x->st_out = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(x->status) + kStatusBytes);
   }
   if (ok && (c.flags & SMETRIC_FLAG_PIPELINE)) ok = pipeline_attach(x) == SMETRIC_OK;
   if (ok) ok = kernel_limits(x) && cudaMemset(x->table, 0, table_bytes) == cudaSuccess &&

@@ -3409,8 +3409,6 @@ int smetric_route_batch_host(smetric_index* idx, const int32_t* h_tokens, int64_
   int64_t* const d_offsets = idx->st_in + N;
   uint64_t* const d_sk = idx->st_out;
   int32_t* const o = reinterpret_cast<int32_t*>(idx->st_out + R);
-  unsigned char* const pin_out = idx->st_pin;
-  int32_t* const pin_status = reinterpret_cast<int32_t*>(pin_out + kHostPinOut);
   // The caller's arrays are read when the stream gets there: pinned ones may still be written by what is enqueued
   // before this call.
   bool ok = true;
@@ -3424,18 +3422,18 @@ int smetric_route_batch_host(smetric_index* idx, const int32_t* h_tokens, int64_
                            d_sk, nullptr, 0, stream);
   if (rc) return rc;
   if (small) {
-    // every output and the status, then one wait
-    ok = cudaMemcpyAsync(pin_out, idx->st_out, R * 20, cudaMemcpyDeviceToHost, s) == cudaSuccess &&
-         cudaMemcpyAsync(pin_status, idx->status, sizeof(int32_t), cudaMemcpyDeviceToHost, s) == cudaSuccess;
+    // the status and every output, then one wait
+    ok = cudaMemcpyAsync(idx->st_pin, idx->status, kStatusBytes + R * 20, cudaMemcpyDeviceToHost, s) == cudaSuccess;
     if (cudaStreamSynchronize(s) != cudaSuccess || !ok) return cuda_status(cudaErrorUnknown);
-    memcpy(h_session_key, pin_out, R * sizeof(uint64_t));
-    const unsigned char* const p = pin_out + R * sizeof(uint64_t);
+    const int32_t status = *reinterpret_cast<const int32_t*>(idx->st_pin);
+    const unsigned char* const keys = idx->st_pin + kStatusBytes;
+    const unsigned char* const p = keys + R * sizeof(uint64_t);
+    memcpy(h_session_key, keys, R * sizeof(uint64_t));
     memcpy(h_instance, p, R * sizeof(int32_t));
     memcpy(h_local_hit, p + R * sizeof(int32_t), R * sizeof(int32_t));
     memcpy(h_global_hit, p + 2 * R * sizeof(int32_t), R * sizeof(int32_t));
-    if (*pin_status != 0 && cudaMemset(idx->status, 0, sizeof(int32_t)) != cudaSuccess)
-      return cuda_status(cudaErrorUnknown);
-    return *pin_status;
+    if (status != 0 && cudaMemset(idx->status, 0, sizeof(int32_t)) != cudaSuccess) return cuda_status(cudaErrorUnknown);
+    return status;
   }
   ok = cudaMemcpyAsync(h_instance, o, R * sizeof(int32_t), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
        cudaMemcpyAsync(h_local_hit, o + R, R * sizeof(int32_t), cudaMemcpyDeviceToHost, s) == cudaSuccess &&

@@ -97,16 +97,16 @@ __host__ __device__ constexpr int entry_words(int W) { return W == 1 ? 2 : (W <=
 // and probe in one kernel) and the chain alone in the calls that only hash.
 enum RouteKernel { kPrep = 0, kDigest = 1, kChainProbe = 2, kWalk = 3, kNumRouteKernels = 4 };
 
-// smetric_route_batch_host: the outputs and the status of batches of up to this
-// many requests come back in two copies to the index's pinned buffer and one
-// wait. (Longer ones are copied to the caller's arrays: the extra pass over 20
-// bytes a request costs the host more than the copies saved.) Inputs are always
-// copied from the caller's arrays, in stream order. 16 requests of 6,000 tokens:
-// 83 us a call, 98 with four copies down and the status read by a synchronous
-// copy of its own.
+// smetric_route_batch_host: the status and the outputs of batches of up to this
+// many requests come back in one copy to the index's pinned buffer and one wait.
+// (Longer ones are copied to the caller's arrays: the extra pass over 20 bytes a
+// request costs the host more than the copies saved.) Inputs are always copied
+// from the caller's arrays, in stream order. 16 requests of 6,000 tokens: 81 us
+// a call, 83 with a copy of its own for the status, 98 with four copies down
+// and the status read by a synchronous one.
 constexpr int64_t kHostSmall = 2048;
-constexpr size_t kHostPinOut = (size_t)kHostSmall * 20;
-constexpr size_t kHostPin = kHostPinOut + 16;
+constexpr size_t kStatusBytes = 16;  // before the outputs, so that one copy takes both
+constexpr size_t kHostPin = kStatusBytes + (size_t)kHostSmall * 20;
 
 struct ProfileSlot {
   cudaEvent_t ev[kNumRouteKernels + 1];
@@ -169,8 +169,8 @@ struct smetric_index {
   // staging for smetric_route_batch_host
   int32_t* st_tokens;
   int64_t* st_in;       // num_instances loads, then max_batch_requests + 1 offsets
-  uint64_t* st_out;     // a batch's session keys, then its 3 n int32 outputs (20 bytes a request)
-  unsigned char* st_pin;  // pinned host memory: kHostSmall requests' outputs, and the status
+  uint64_t* st_out;     // after the status word: a batch's session keys, then its 3 n int32 outputs (20 bytes a request)
+  unsigned char* st_pin;  // pinned host memory: the status, and kHostSmall requests' outputs
   int digest_occ;  // resident digest CTAs per SM (0 until the first route)
   smetric::LruState* lru;  // capped tiers' recency (NULL: no tier capped)
   // observability
